@@ -854,12 +854,12 @@ int run_residual(fftm_problem* p, int slot, bool test_outputs, bool solver_form 
   int blocks = 0;
   ProfScope ps(p, test_outputs ? FFTM_KCAT_OTHER : FFTM_KCAT_RESIDUAL);
   CU(launch_residual<T>(R, p->tetra, test_outputs, p->ctx->stream, &blocks));
-  CU(launch_reduce_norms(p->partial, blocks, 2, p->dscal, p->ctx->stream, p->stop));
+  if (p->stop && !test_outputs && !solver_form)  // with the convergence test on the device
+    CU(launch_check(p->partial, blocks, p->dscal, p->dctl, p->derr, p->desc.tol, p->desc.max_iter, p->h[0],
+                    p->ctx->stream));
+  else
+    CU(launch_norms(p->partial, blocks, p->dscal, false, p->h[0], p->ctx->stream, p->stop));
   p->launches += 2;
-  if (p->stop && !test_outputs && !solver_form) {  // the convergence test on the device
-    CU(launch_check(p->dscal, p->dctl, p->derr, p->desc.tol, p->desc.max_iter, p->h[0], p->ctx->stream));
-    p->launches += 1;
-  }
   return FFTM_OK;
 }
 
@@ -1306,7 +1306,7 @@ int solve_step_t(fftm_problem* p, fftm_step_report* rep, double* err_hist, int* 
       ResParams<T> R = res_params<T>(p, sm, nullptr, nullptr);
       ProfScope ps(p, FFTM_KCAT_OTHER);
       CU(launch_stats<T>(R, p->tetra, p->partial, kStatsBlocks, s));
-      CU(launch_reduce_norms(p->partial, kStatsBlocks, 18, p->dscal + 16, s));
+      CU(launch_reduce_sums(p->partial, kStatsBlocks, 18, p->dscal + 16, s));
       p->launches += 2;
     }
     CU(cudaMemcpyAsync(p->hpin, p->dscal, (mixed ? 25 : 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1355,7 +1355,7 @@ int solve_step_t(fftm_problem* p, fftm_step_report* rep, double* err_hist, int* 
     ResParams<T> R = res_params<T>(p, p->cur, nullptr, nullptr);
     ProfScope ps(p, FFTM_KCAT_OTHER);
     CU(launch_stats<T>(R, p->tetra, p->partial, sb, s));
-    CU(launch_reduce_norms(p->partial, sb, 18, p->dscal + 16, s));
+    CU(launch_reduce_sums(p->partial, sb, 18, p->dscal + 16, s));
     p->launches += 2;
   }
   CU(cudaMemcpyAsync(p->hpin + 16, p->dscal + 16, 18 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2712,13 +2712,6 @@ int noalloc_scratch(int device, double** out) {
   return FFTM_OK;
 }
 
-__global__ void k_noalloc_norms(const double* __restrict__ sums, double h1, double* __restrict__ norms) {
-  const double sd = sums[0], sp = sums[1];
-  norms[0] = sd;
-  norms[1] = sp;
-  norms[2] = sp > 0.0 ? h1 * sqrt(sd / sp) : (sd == 0.0 ? 0.0 : CUDART_INF);
-}
-
 template <typename T>
 int residual_noalloc_t(fftm_problem* p, const T* u, T* D, double* norms) {
   double* scratch = nullptr;
@@ -2741,13 +2734,10 @@ int residual_noalloc_t(fftm_problem* p, const T* u, T* D, double* norms) {
                                            " doubles; the maximum is " +
                                            std::to_string(kNoAllocScratchDoubles - 4) + ")");
   R.partial = scratch;  // every block overwrites its two slots: nothing has to start at zero
-  double* sums = scratch + kNoAllocScratchDoubles - 4;
   cudaStream_t s = p->ctx->stream;
   CU(launch_residual<T>(R, p->tetra, false, s, nullptr));
-  CU(launch_reduce_norms(scratch, blocks, 2, sums, s));
-  k_noalloc_norms<<<1, 1, 0, s>>>(sums, p->h[0], norms);
-  CU(cudaGetLastError());
-  p->launches += 3;
+  CU(launch_norms(scratch, blocks, norms, true, p->h[0], s));
+  p->launches += 2;
   return FFTM_OK;
 }
 

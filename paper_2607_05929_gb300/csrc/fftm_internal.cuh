@@ -275,14 +275,20 @@ cudaError_t launch_commit(const ResParams<T>& P, int tetra, T* out, cudaStream_t
 template <typename T>
 cudaError_t launch_state_io(const ResParams<T>& P, int tetra, T* out, const T* in, cudaStream_t s);
 
-cudaError_t launch_reduce_norms(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
-                                const int* stop = nullptr);
+// out[v] = sum over the rows of partial[row * nvals + v]
+cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
+                               const int* stop = nullptr);
+// S_D and S_P of the residual's block partials (rows of two, 16-byte aligned) -> sums[0..1] and,
+// with err_too, err = h1 sqrt(S_D / S_P) -> sums[2]
+cudaError_t launch_norms(const double* partial, int nblocks, double* sums, bool err_too, double h1, cudaStream_t s,
+                         const int* stop = nullptr);
 // Control block of a load step whose convergence is decided on the device (Algorithm 1's
 // test, Eq. equilibrium_condition): ctl[0] stop (0 running, 1 converged, 2 diverged,
 // 3 iteration limit), ctl[1] the iteration to check next, ctl[2] the iteration checked last.
-// k_check reads S_D, S_P from sums, records err at err_hist[m] and stops the step or moves on.
-cudaError_t launch_check(const double* sums, int* ctl, double* err_hist, double tol, int max_iter, double h1,
-                         cudaStream_t s);
+// k_check sums the partials as launch_norms does (-> sums), records err at err_hist[m] and stops
+// the step or moves on.
+cudaError_t launch_check(const double* partial, int nblocks, double* sums, int* ctl, double* err_hist, double tol,
+                         int max_iter, double h1, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_axpy_fields(T* const dst[3], const T* const a[3], const T* const b[3], T alpha,

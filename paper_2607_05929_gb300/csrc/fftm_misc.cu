@@ -14,56 +14,112 @@
 // times its diagonal entry rejects the step (c = e_last).
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "fftm_internal.cuh"
 
 namespace fftm {
 
-// Sum `nvals` doubles over `nblocks` rows (fixed order: deterministic).
+// Sum `nvals` doubles over `nblocks` rows (fixed order: deterministic).  One warp per column:
+// FP64 adds issue at one warp instruction in 16 cycles per SM here, so the sums are arranged
+// for few of them (a lane's rows, then five shuffles per column).
 __global__ void k_reduce(const double* __restrict__ partial, int nblocks, int nvals, double* __restrict__ out,
                          const int* __restrict__ stop) {
   if (stop && *stop) return;
-  __shared__ double red[256];
-  for (int v = 0; v < nvals; ++v) {
+  const int lane = threadIdx.x & 31;
+  for (int v = threadIdx.x >> 5; v < nvals; v += blockDim.x >> 5) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[(size_t)b * nvals + v];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[v] = red[0];
-    __syncthreads();
+#pragma unroll 4
+    for (int b = lane; b < nblocks; b += 32) s += partial[(size_t)b * nvals + v];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) out[v] = s;
   }
 }
 
-cudaError_t launch_reduce_norms(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
-                                const int* stop) {
-  k_reduce<<<1, 256, 0, s>>>(partial, nblocks, nvals, out, stop);
+// S_D and S_P over the residual's block partials (rows of two), in one block: NORM_THREADS
+// threads read a row at a time, several in flight; valid in thread 0.
+constexpr int NORM_THREADS = 256;
+__device__ __forceinline__ double2 norm_sums(const double* __restrict__ partial, int nblocks) {
+  __shared__ double2 red[NORM_THREADS / 32];
+  const double2* rows = reinterpret_cast<const double2*>(partial);
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int b = threadIdx.x; b < nblocks; b += NORM_THREADS) {
+    const double2 r = rows[b];
+    s.x += r.x;
+    s.y += r.y;
+  }
+  const int lane = threadIdx.x & 31;
+  for (int off = 16; off > 0; off >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+  }
+  if (lane == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < NORM_THREADS / 32; ++w) {
+      s.x += red[w].x;
+      s.y += red[w].y;
+    }
+  return s;
+}
+
+// err = h1 sqrt(S_D / S_P) (Eq. equilibrium_condition; +inf while S_P is 0 under a non-zero S_D)
+__device__ __forceinline__ double norm_error(double2 s, double h1) {
+  return s.y > 0.0 ? h1 * sqrt(s.x / s.y) : (s.x == 0.0 ? 0.0 : CUDART_INF);
+}
+
+// sums[0..1] = S_D, S_P and, with err_too, sums[2] = err
+__global__ void __launch_bounds__(NORM_THREADS) k_norms(const double* __restrict__ partial, int nblocks,
+                                                        double* __restrict__ sums, int err_too, double h1,
+                                                        const int* __restrict__ stop) {
+  if (stop && *stop) return;
+  const double2 s = norm_sums(partial, nblocks);
+  if (threadIdx.x != 0) return;
+  sums[0] = s.x;
+  sums[1] = s.y;
+  if (err_too) sums[2] = norm_error(s, h1);
+}
+
+cudaError_t launch_norms(const double* partial, int nblocks, double* sums, bool err_too, double h1, cudaStream_t s,
+                         const int* stop) {
+  k_norms<<<1, NORM_THREADS, 0, s>>>(partial, nblocks, sums, err_too ? 1 : 0, h1, stop);
   return cudaGetLastError();
 }
 
-// The convergence test of Algorithm 1 on the device: err = h1 sqrt(S_D / S_P) (Eq.
-// equilibrium_condition; +inf while S_P is 0 under a non-zero S_D, which only means "not yet"),
-// recorded at err_hist[m]; the step stops when err < tol (1), on a non-finite norm (2) or at the
-// iteration limit (3), else the next iteration is m + 1.
-__global__ void k_check(const double* __restrict__ sums, int* __restrict__ ctl, double* __restrict__ err_hist,
-                        double tol, int max_iter, double h1) {
+cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
+                               const int* stop) {
+  k_reduce<<<1, 32 * (nvals < 32 ? nvals : 32), 0, s>>>(partial, nblocks, nvals, out, stop);
+  return cudaGetLastError();
+}
+
+// The norms and the convergence test of Algorithm 1 on the device, in one launch (the sum of
+// the partials and the test were two: 10 + 4 us per iteration, now 5 with the same sums): err
+// (Eq. equilibrium_condition; +inf only means "not yet") is recorded at err_hist[m]; the step
+// stops when err < tol (1), on a non-finite norm (2) or at the iteration limit (3), else the
+// next iteration is m + 1.
+__global__ void __launch_bounds__(NORM_THREADS) k_check(const double* __restrict__ partial, int nblocks,
+                                                        double* __restrict__ sums, int* __restrict__ ctl,
+                                                        double* __restrict__ err_hist, double tol, int max_iter,
+                                                        double h1) {
   if (ctl[0]) return;
+  const double2 s = norm_sums(partial, nblocks);
+  if (threadIdx.x != 0) return;
   const int m = ctl[1];
-  const double sd = sums[0], sp = sums[1];
-  const double err = sp > 0.0 ? h1 * sqrt(sd / sp) : (sd == 0.0 ? 0.0 : CUDART_INF);
+  const double err = norm_error(s, h1);
+  sums[0] = s.x;
+  sums[1] = s.y;
   err_hist[m] = err;
   ctl[2] = m;
-  if (isnan(err) || isinf(sd) || isinf(sp) || isnan(sd) || isnan(sp)) ctl[0] = 2;
+  if (isnan(err) || isinf(s.x) || isinf(s.y) || isnan(s.x) || isnan(s.y)) ctl[0] = 2;
   else if (err < tol) ctl[0] = 1;
   else if (m >= max_iter) ctl[0] = 3;
   else ctl[1] = m + 1;
 }
 
-cudaError_t launch_check(const double* sums, int* ctl, double* err_hist, double tol, int max_iter, double h1,
-                         cudaStream_t s) {
-  k_check<<<1, 1, 0, s>>>(sums, ctl, err_hist, tol, max_iter, h1);
+cudaError_t launch_check(const double* partial, int nblocks, double* sums, int* ctl, double* err_hist, double tol,
+                         int max_iter, double h1, cudaStream_t s) {
+  k_check<<<1, NORM_THREADS, 0, s>>>(partial, nblocks, sums, ctl, err_hist, tol, max_iter, h1);
   return cudaGetLastError();
 }
 
@@ -101,10 +157,9 @@ cudaError_t launch_axpy_fields(T* const dst[3], const T* const a[3], const T* co
   return cudaGetLastError();
 }
 
-int gram_blocks(long long count) {
-  (void)count;
-  return 152 * 4;
-}
+// Four blocks per SM, and no more than one element per thread needs: a block ends with 9 FP64
+// warp sums whatever it read (at 32^3 608 blocks took 22 us, 148 take 9).
+int gram_blocks(long long count) { return (int)std::min<long long>(152 * 4, (count + 255) / 256); }
 
 // Normal matrix of the residual differences d_k = D_k - D_last (k < last) and
 // the right-hand side <d_k, D_last>, formed from explicit differences (no
@@ -195,18 +250,24 @@ cudaError_t launch_gram(const T* const D[4][3], int m, long long count, double* 
   return cudaGetLastError();
 }
 
-// Reduce the partials; solve (d^T d) gamma = -(d^T D_last) by Cholesky in FP64;
+// Reduce the partials (one warp per sum, its rows in flight together: a single warp that walked
+// them in a chain of dependent loads took 49-57 us at any grid size, this takes 6); solve
+// (d^T d) gamma = -(d^T D_last) by Cholesky in FP64;
 // c_k = gamma_k (k < last), c_last = 1 - sum gamma.  A pivot below pivot_tol
 // times its diagonal entry rejects the step: c = e_last.
-__global__ void k_anderson_solve(const double* __restrict__ partial, int nblocks, int m, double pivot_tol,
-                                 double* __restrict__ coef, int* __restrict__ accepted, const int* __restrict__ ctl) {
+__global__ void __launch_bounds__(288) k_anderson_solve(const double* __restrict__ partial, int nblocks, int m,
+                                                        double pivot_tol, double* __restrict__ coef,
+                                                        int* __restrict__ accepted, const int* __restrict__ ctl) {
   if (ctl && ctl[0]) return;
   if (ctl) accepted += ctl[2];
   __shared__ double g[9];
-  if (threadIdx.x < 9) {
+  {
+    const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += partial[(size_t)b * 9 + threadIdx.x];
-    g[threadIdx.x] = t;
+#pragma unroll 8
+    for (int b = lane; b < nblocks; b += 32) t += partial[(size_t)b * 9 + v];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (lane == 0) g[v] = t;
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -257,7 +318,7 @@ __global__ void k_anderson_solve(const double* __restrict__ partial, int nblocks
 
 cudaError_t launch_anderson_solve(const double* partial, int nblocks, int m, double pivot_tol, double* coef,
                                   int* accepted, cudaStream_t s, const int* ctl) {
-  k_anderson_solve<<<1, 32, 0, s>>>(partial, nblocks, m, pivot_tol, coef, accepted, ctl);
+  k_anderson_solve<<<1, 288, 0, s>>>(partial, nblocks, m, pivot_tol, coef, accepted, ctl);
   return cudaGetLastError();
 }
 

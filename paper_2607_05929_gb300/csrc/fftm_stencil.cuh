@@ -749,6 +749,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // fixed number of blocks, so the per-block FP64 partials (S_D from k_div, S_P
 // from k_stress, same block index) have a bounded count.
 constexpr int RTX = 32, RTY = 8, RBLOCKS = 2432;
+constexpr int kFaceBlocks = 152 * 8;  // a few node components per thread at 256^3 (each a chain of gathers)
 
 // Tiles of RTX x RTY (x, y) positions of one z plane over the box [o, o + e).
 struct TileIdx {
@@ -1123,9 +1124,14 @@ __device__ __forceinline__ T store_node(const ResParams<T>& P, int mx, int my, i
   return sdn;
 }
 
-// Interior nodes: all 8 neighbouring voxels exist (or wrap); plain differences.
+// Blocks [0, nbf) take the face nodes (each once, with the ghost rules), the others the
+// interior ones, where all 8 neighbouring voxels exist (or wrap): plain differences.  A face
+// node is a chain of index arithmetic and 24 gathers per component, bound by its latency, so
+// each thread takes one component of one node and the chains run beside the interior's
+// (43 -> 16 us at 32^3 in FP64, where a thread used to walk an interior node and then a face
+// node with its three components in turn).
 template <typename T, int TETRA, bool WITH_P, bool SYM, bool INC>
-__global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi) {
+__global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
   if (P.stop && *P.stop) return;
   constexpr int NC = SYM ? 6 : 9;
   constexpr int NCT = WITH_P ? NC + 9 : NC;
@@ -1136,7 +1142,26 @@ __global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, F
   T sd = T(0);
   double SD = 0.0;
   int run = 0;
-  for (int t = blockIdx.x; t < ti.ntile; t += gridDim.x) {
+  if ((int)blockIdx.x < nbf) {
+    int nface[3] = {n1, n2, n3};
+    const int total = 3 * fi.count;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += nbf * blockDim.x) {
+      const int q = t / fi.count;
+      int m[3];
+      if (!fi.at(t - q * fi.count, nface, m)) continue;
+      const bool dof = m[0] >= P.lo[q][0] && m[0] < P.hi[q][0] && m[1] >= P.lo[q][1] && m[1] < P.hi[q][1] &&
+                       m[2] >= P.lo[q][2] && m[2] < P.hi[q][2];
+      T Dq[3] = {T(0), T(0), T(0)}, pq[3] = {T(0), T(0), T(0)};
+      if (dof) node_div_general<T, TETRA, WITH_P, SYM>(P, m[0], m[1], m[2], Dq, pq, 1 << q);
+      const int off = m[0] + m[1] * (int)P.sy + m[2] * (int)P.sz;
+      const T d = (INC && dof) ? Dq[q] + __ldg(P.Dn[q] + off) : Dq[q];
+      P.D[q][off] = dof ? d : T(0);
+      if (WITH_P) P.p[q][off] = dof ? pq[q] : T(0);
+      if (dof) SD += (double)(d * d);
+    }
+  }
+  const int ntile = (int)blockIdx.x < nbf ? 0 : ti.ntile, step = (int)gridDim.x - nbf;
+  for (int t = max(0, (int)blockIdx.x - nbf); t < ntile; t += step) {
     int x0, y0, mz;
     ti.at(t, &x0, &y0, &mz);
     const int mx = x0 + (threadIdx.x % RTX), my = y0 + (threadIdx.x / RTX);
@@ -1188,15 +1213,6 @@ __global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, F
       sd = T(0);
       run = 0;
     }
-  }
-  // face nodes, each once, with the ghost rules
-  int nface[3] = {n1, n2, n3};
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < fi.count; t += gridDim.x * blockDim.x) {
-    int m[3];
-    if (!fi.at(t, nface, m)) continue;
-    T Dq[3] = {T(0), T(0), T(0)}, pq[3] = {T(0), T(0), T(0)};
-    node_div_general<T, TETRA, WITH_P, SYM>(P, m[0], m[1], m[2], Dq, pq);
-    SD += (double)store_node<T, WITH_P, INC>(P, m[0], m[1], m[2], Dq, pq);
   }
   SD += (double)sd;
   const double tot = block_sum(SD, red);
@@ -1730,8 +1746,6 @@ __global__ void __launch_bounds__(256, 2) k_face_div(ResParams<T> P, FaceIdx fi)
   }
 }
 
-constexpr int kFaceBlocks = 152 * 8;  // a few node components per thread at 256^3 (each a chain of gathers)
-
 template <typename T>
 static size_t fused_smem(int tetra, int fy) {
   using NVs = typename NodeV<T, true>::t;  // same size as the FP64 node value
@@ -1796,10 +1810,28 @@ static cudaError_t launch_fused_t(const ResParams<T>& P, cudaStream_t s, int* bl
   return cudaSuccess;
 }
 
+// Blocks of the two-pass form: at most RBLOCKS (16 per SM) over the interior or the voxels, no
+// more than there are tiles -- an empty block still pays its FP64 block sum, and the norm
+// reduction one row (at 32^3 only 128 of 2432 had a tile) -- plus k_div's face blocks.  Both
+// kernels get the same count (one S_D and one S_P slot per block).
+template <typename T>
+static int face_blocks(const FaceIdx& fi) {
+  return std::min(kFaceBlocks, (3 * fi.count + RTX * RTY - 1) / (RTX * RTY));
+}
+
+template <typename T>
+static int two_pass_blocks(const ResParams<T>& P) {
+  const TileIdx tv = voxel_tiles(P.n);
+  TileIdx tn;
+  FaceIdx fi;
+  interior_and_faces<T>(P, &tn, &fi);
+  return std::max(std::min(RBLOCKS, tv.ntile), face_blocks<T>(fi) + std::min(RBLOCKS, std::max(1, tn.ntile)));
+}
+
 template <typename T>
 int residual_blocks(const ResParams<T>& P, int tetra) {
   (void)tetra;
-  return fused_ok(P, false) ? fused_blocks(P) : RBLOCKS;
+  return fused_ok(P, false) ? fused_blocks(P) : two_pass_blocks(P);
 }
 
 template <typename T, int TETRA, bool WITH_P, bool SYM>
@@ -1808,30 +1840,31 @@ static cudaError_t launch_res_t(const ResParams<T>& P, bool lo, cudaStream_t s, 
   TileIdx tn;
   FaceIdx fi;
   interior_and_faces<T>(P, &tn, &fi);
+  const int nb = two_pass_blocks(P), nbf = face_blocks<T>(fi);
   const bool inc = !WITH_P && P.inc;
   if (inc) {
-    if (lo) k_stress_inc<T, TETRA, true, SYM><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
-    else k_stress_inc<T, TETRA, false, SYM><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
+    if (lo) k_stress_inc<T, TETRA, true, SYM><<<nb, RTX * RTY, 0, s>>>(P, tv);
+    else k_stress_inc<T, TETRA, false, SYM><<<nb, RTX * RTY, 0, s>>>(P, tv);
   } else {
     if (P.slaw == 1) {
-      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 1><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
-      else k_stress<T, TETRA, WITH_P, false, SYM, 1><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
+      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 1><<<nb, RTX * RTY, 0, s>>>(P, tv);
+      else k_stress<T, TETRA, WITH_P, false, SYM, 1><<<nb, RTX * RTY, 0, s>>>(P, tv);
     } else if (P.slaw == 2) {
-      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 2><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
-      else k_stress<T, TETRA, WITH_P, false, SYM, 2><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
+      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 2><<<nb, RTX * RTY, 0, s>>>(P, tv);
+      else k_stress<T, TETRA, WITH_P, false, SYM, 2><<<nb, RTX * RTY, 0, s>>>(P, tv);
     } else if (P.slaw == 4) {
-      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 4><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
-      else k_stress<T, TETRA, WITH_P, false, SYM, 4><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
+      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 4><<<nb, RTX * RTY, 0, s>>>(P, tv);
+      else k_stress<T, TETRA, WITH_P, false, SYM, 4><<<nb, RTX * RTY, 0, s>>>(P, tv);
     } else {
-      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 0><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
-      else k_stress<T, TETRA, WITH_P, false, SYM, 0><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tv);
+      if (lo) k_stress<T, TETRA, WITH_P, true, SYM, 0><<<nb, RTX * RTY, 0, s>>>(P, tv);
+      else k_stress<T, TETRA, WITH_P, false, SYM, 0><<<nb, RTX * RTY, 0, s>>>(P, tv);
     }
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (inc) k_div<T, TETRA, false, SYM, true><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tn, fi);
-  else k_div<T, TETRA, WITH_P, SYM, false><<<RBLOCKS, RTX * RTY, 0, s>>>(P, tn, fi);
-  if (blocks_out) *blocks_out = RBLOCKS;
+  if (inc) k_div<T, TETRA, false, SYM, true><<<nb, RTX * RTY, 0, s>>>(P, tn, fi, nbf);
+  else k_div<T, TETRA, WITH_P, SYM, false><<<nb, RTX * RTY, 0, s>>>(P, tn, fi, nbf);
+  if (blocks_out) *blocks_out = nb;
   return cudaGetLastError();
 }
 
