@@ -1623,8 +1623,8 @@ static int set_load_field_t(fftm_problem* p, const void* u, int is_device, size_
   }
   T* dst[3];
   for (int q = 0; q < 3; ++q) dst[q] = reinterpret_cast<T*>(p->ustar) + q * p->comp_stride;
-  CU(launch_pack<T>((const T* const*)dst, const_cast<T*>(reinterpret_cast<const T*>(from)), p->N[0], p->N[1],
-                    p->N[2], p->sy, p->sz, 1, s));
+  CU(launch_unpack<T>(dst, reinterpret_cast<const T*>(from), p->N[0], p->N[1], p->N[2], p->sy, p->sz, nullptr,
+                      nullptr, s));
   CU(cudaStreamSynchronize(s));
   p->launches++;
   return FFTM_OK;
@@ -2441,7 +2441,7 @@ static int get_field_t(fftm_problem* p, int field, void* dst, int dst_is_device,
         src[q] = field_ptr<T>(p, field == FFTM_FIELD_U ? SET_UH + p->cur : SET_WORK, q);
       }
     }
-    CU(launch_pack<T>(src, reinterpret_cast<T*>(target), p->N[0], p->N[1], p->N[2], p->sy, p->sz, 0, s));
+    CU(launch_pack<T>(src, reinterpret_cast<T*>(target), p->N[0], p->N[1], p->N[2], p->sy, p->sz, s));
   } else {
     ResParams<T> R = res_params<T>(p, p->cur, nullptr, nullptr);
     T* g = field == FFTM_FIELD_GRAD ? reinterpret_cast<T*>(target) : nullptr;
@@ -2484,10 +2484,9 @@ static int set_field_t(fftm_problem* p, int field, const void* src, int src_is_d
   if (field == FFTM_FIELD_U && p->esz == 4)
     for (int q = 0; q < 3; ++q)
       CU(cudaMemsetAsync(field_ptr<T>(p, SET_UL + p->cur, q), 0, p->comp_stride * sizeof(T), s));
-  CU(launch_pack<T>((const T* const*)dst, const_cast<T*>(reinterpret_cast<const T*>(from)), p->N[0], p->N[1],
-                    p->N[2], p->sy, p->sz, 1, s));
-  CU(launch_mask<T>(dst, p->lo, p->hi, p->N[0], p->N[1], p->N[2], p->sy, p->sz, s));
-  p->launches += 2;
+  CU(launch_unpack<T>(dst, reinterpret_cast<const T*>(from), p->N[0], p->N[1], p->N[2], p->sy, p->sz, p->lo, p->hi,
+                      s));
+  p->launches++;
   CU(cudaStreamSynchronize(s));
   return FFTM_OK;
 }

@@ -311,12 +311,14 @@ cudaError_t launch_combine(T* const dst[3], T* const bh[3], T* const bl[3], cons
                            long long count, cudaStream_t s, const int* stop = nullptr);
 template <typename T>
 cudaError_t launch_voxel_fields(const ResParams<T>& P, int tetra, T* grad_out, T* stress_out, cudaStream_t s);
+// Dense [q][z][y][x] <-> pitched component arrays; unpack stores zero outside [lo, hi) (null: the
+// whole range).
 template <typename T>
-cudaError_t launch_pack(const T* const src[3], T* dst, int N1, int N2, int N3, long long sy, long long sz,
-                        int unpack, cudaStream_t s);
+cudaError_t launch_pack(const T* const src[3], T* dense, int N1, int N2, int N3, long long sy, long long sz,
+                        cudaStream_t s);
 template <typename T>
-cudaError_t launch_mask(T* const f[3], const int lo[3][3], const int hi[3][3], int N1, int N2, int N3,
-                        long long sy, long long sz, cudaStream_t s);
+cudaError_t launch_unpack(T* const dst[3], const T* dense, int N1, int N2, int N3, long long sy, long long sz,
+                          const int (*lo)[3], const int (*hi)[3], cudaStream_t s);
 
 int gram_blocks(long long count);
 // Measured FMA throughput of the current device (FLOP/s, an FMA counting two), FP64 or FP32.
