@@ -1031,7 +1031,6 @@ double error_of(fftm_problem* p, double SD, double SP) {
 // increment -(C0_FF)^-1 <sigma>_F of the isotropic reference stiffness restricted to the
 // free components (the normal ones couple through lambda0, the shear ones decouple).
 constexpr int kVoigt[6][2] = {{0, 0}, {1, 1}, {2, 2}, {1, 2}, {0, 2}, {0, 1}};
-constexpr int kStatsBlocks = 152 * 2;  // blocks of the mean stress / strain reduction
 
 void mixed_increment(const double sig[3][3], int mask, double lam0, double mu0, double d[3][3]) {
   for (int i = 0; i < 3; ++i)
@@ -1305,8 +1304,12 @@ int solve_step_t(fftm_problem* p, fftm_step_report* rep, double* err_hist, int* 
     if (mixed) {  // the mean stress of this iterate (voxel points)
       ResParams<T> R = res_params<T>(p, sm, nullptr, nullptr);
       ProfScope ps(p, FFTM_KCAT_OTHER);
-      CU(launch_stats<T>(R, p->tetra, p->partial, kStatsBlocks, s));
-      CU(launch_reduce_sums(p->partial, kStatsBlocks, 18, p->dscal + 16, s));
+      // the plain two-pass residual has left every point's stress in vs; else evaluate the law again
+      int sb = 0;
+      const bool stored = p->res_two_pass > 0 && !p->committed;
+      if (stored) CU(launch_stress_sums<T>(R, p->tetra, p->partial, &sb, s));
+      else CU(launch_stats<T>(R, p->tetra, p->partial, &sb, s));
+      CU(launch_reduce_sums(p->partial, sb, stored ? 9 : 18, p->dscal + 16, s));
       p->launches += 2;
     }
     CU(cudaMemcpyAsync(p->hpin, p->dscal, (mixed ? 25 : 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1350,11 +1353,11 @@ int solve_step_t(fftm_problem* p, fftm_step_report* rep, double* err_hist, int* 
     std::memcpy(p->mixed_A, p->load.A, sizeof(p->mixed_A));
     p->mixed_prev = p->load.mixed;
   }
-  const int sb = kStatsBlocks;
   {
     ResParams<T> R = res_params<T>(p, p->cur, nullptr, nullptr);
     ProfScope ps(p, FFTM_KCAT_OTHER);
-    CU(launch_stats<T>(R, p->tetra, p->partial, sb, s));
+    int sb = 0;
+    CU(launch_stats<T>(R, p->tetra, p->partial, &sb, s));
     CU(launch_reduce_sums(p->partial, sb, 18, p->dscal + 16, s));
     p->launches += 2;
   }

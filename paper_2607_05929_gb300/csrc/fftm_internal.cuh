@@ -344,7 +344,11 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // wait until at most one committed group is still in flight
 __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+// Sums over the voxel points: rows of 18 (P[3 i + q], then G[3 i + q]), their count in *nblocks.
 template <typename T>
-cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int nblocks, cudaStream_t s);
+cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s);
+// The same for P alone (rows of 9), from the stresses that a plain two-pass residual left in P.vs.
+template <typename T>
+cudaError_t launch_stress_sums(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s);
 
 }  // namespace fftm

@@ -1891,68 +1891,86 @@ bool residual_one_pass(const ResParams<T>& P) {
 }
 
 // ---- per-voxel evaluation shared by the output and statistics kernels ----
-template <typename T, int TETRA, bool LO>
-__device__ __forceinline__ int voxel_eval(const ResParams<T>& P, long long v, T Gt_out[2][9], T P_out[2][9],
+// SL: the law with internal variables that the problem holds (as ResParams::slaw), so that a
+// kernel carries the registers of that law alone: with crystal plasticity compiled into every
+// instance an elastic problem's k_stats had 255 registers and spilled (3.4 ms at 256^3).
+template <typename T, int TETRA, bool LO, int SL>
+__device__ __forceinline__ int voxel_eval(const ResParams<T>& P, int vx, int vy, int vz, T Gt_out[2][9], T P_out[2][9],
                                           T (*stn)[10] = nullptr) {
   const int n1 = P.n[0], n2 = P.n[1], n3 = P.n[2];
-  const int vx = (int)(v % n1);
-  const long long r1 = v / n1;
-  const int vy = (int)(r1 % n2);
-  const int vz = (int)(r1 / n2);
-  const int ph = P.phase[vx + vy * P.vy + (long long)vz * P.vz];
+  const long long nvox = (long long)n1 * n2 * n3;
+  const long long v = vx + vy * P.vy + (long long)vz * P.vz;
+  const int ph = P.phase[v];
   const int law = __ldg(P.law_id + ph);
-  const bool j2 = law == LAW_J2;
+  const bool j2 = (SL & 1) && law == LAW_J2;
   const T* lc = P.law_c + (size_t)ph * LAWC;
-  T uh[3][8], ul[3][8], nh[3][8], nl[3][8];
+  T uh[3][8], ul[3][8];
+  long long at[8];
 #pragma unroll
   for (int o = 0; o < 8; ++o) {
     int gx = vx + (o & 1), gy = vy + ((o >> 1) & 1), gz = vz + (o >> 2);
     if (P.periodic[0] && gx == n1) gx = 0;
     if (P.periodic[1] && gy == n2) gy = 0;
     if (P.periodic[2] && gz == n3) gz = 0;
-    const long long at = gx + gy * P.sy + (long long)gz * P.sz;
+    at[o] = gx + gy * P.sy + (long long)gz * P.sz;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      uh[c][o] = P.u[c][at];
-      ul[c][o] = LO ? P.ulo[c][at] : T(0);
-      nh[c][o] = j2 ? P.un[c][at] : T(0);
-      nl[c][o] = (j2 && LO) ? P.unlo[c][at] : T(0);
+      uh[c][o] = __ldg(P.u[c] + at[o]);
+      ul[c][o] = LO ? __ldg(P.ulo[c] + at[o]) : T(0);
     }
   }
 #pragma unroll
   for (int r = 0; r < (TETRA ? 2 : 1); ++r) {
     T Gf[9];
     law_grad<T, TETRA, LO>(P, false, uh, ul, r, vx, vy, vz, Gf, Gt_out[r]);  // total gradient (reported)
-    if (j2) {
-      T du[3][8], dl[3][8], Gd[9], Ginc[9];
+    if (!j2) point_law<T, SL>(P, law, lc, Gt_out[r], r, v, nvox, P_out[r], stn ? stn[r] : nullptr);
+  }
+  if (j2) {  // from the increment since the commit
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+    for (int o = 0; o < 8; ++o)
 #pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          du[c][o] = uh[c][o] - nh[c][o];
-          dl[c][o] = ul[c][o] - nl[c][o];
-        }
-      law_grad<T, TETRA, LO>(P, true, du, dl, r, vx, vy, vz, Gd, Ginc);
-      point_law<T>(P, law, lc, Ginc, r, v, (long long)n1 * n2 * n3, P_out[r], stn ? stn[r] : nullptr);
-    } else {
-      point_law<T>(P, law, lc, Gt_out[r], r, v, (long long)n1 * n2 * n3, P_out[r], stn ? stn[r] : nullptr);
+      for (int c = 0; c < 3; ++c) {
+        uh[c][o] -= __ldg(P.un[c] + at[o]);
+        if (LO) ul[c][o] -= __ldg(P.unlo[c] + at[o]);
+      }
+#pragma unroll
+    for (int r = 0; r < (TETRA ? 2 : 1); ++r) {
+      T Gd[9], Ginc[9];
+      law_grad<T, TETRA, LO>(P, true, uh, ul, r, vx, vy, vz, Gd, Ginc);
+      point_law<T, SL>(P, law, lc, Ginc, r, v, nvox, P_out[r], stn ? stn[r] : nullptr);
     }
   }
   return law;
 }
 
-template <typename T, int TETRA, bool LO>
-__global__ void k_commit(ResParams<T> P, T* __restrict__ out) {
+// One kernel instance per law with internal variables (K(SL) is a call for that SL).
+#define FFTM_BY_LAW(slaw, K)       \
+  do {                             \
+    if ((slaw) == 1) { K(1); }     \
+    else if ((slaw) == 2) { K(2); }\
+    else if ((slaw) == 4) { K(4); }\
+    else { K(0); }                 \
+  } while (0)
+
+template <typename T, int TETRA, bool LO, int SL>
+__global__ void __launch_bounds__(RTX * RTY) k_commit(ResParams<T> P, TileIdx ti, T* __restrict__ out) {
   const long long nv = (long long)P.n[0] * P.n[1] * P.n[2];
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv;
-       v += (long long)gridDim.x * blockDim.x) {
+  for (int t = blockIdx.x; t < ti.ntile; t += gridDim.x) {
+    int x0, y0, vz;
+    ti.at(t, &x0, &y0, &vz);
+    const int vx = x0 + (threadIdx.x % RTX), vy = y0 + (threadIdx.x / RTX);
+    if (vx >= P.n[0] || vy >= P.n[1]) continue;
+    const long long v = vx + vy * P.vy + (long long)vz * P.vz;
     const int law = __ldg(P.law_id + P.phase[v]);
     if (law != LAW_J2 && law != LAW_CP && law != LAW_LOGJ2) continue;
     T Gt[2][9], Pp[2][9], stn[2][10];
-    voxel_eval<T, TETRA, LO>(P, v, Gt, Pp, stn);
+    voxel_eval<T, TETRA, LO, SL>(P, vx, vy, vz, Gt, Pp, stn);
     const int nc = law == LAW_CP ? 10 : 7;
+#pragma unroll
     for (int r = 0; r < (TETRA ? 2 : 1); ++r)
-      for (int c = 0; c < nc; ++c) out[v + nv * (c + P.nst * r)] = stn[r][c];
+#pragma unroll
+      for (int c = 0; c < 10; ++c)
+        if (c < nc) out[v + nv * (c + P.nst * r)] = stn[r][c];
   }
 }
 
@@ -1960,13 +1978,18 @@ template <typename T>
 cudaError_t launch_commit(const ResParams<T>& P, int tetra, T* out, cudaStream_t s) {
   if (!P.state) return cudaSuccess;
   const bool lo = P.ulo[0] != nullptr;
-  if (tetra) {
-    if (lo) k_commit<T, 1, true><<<1216, 256, 0, s>>>(P, out);
-    else k_commit<T, 1, false><<<1216, 256, 0, s>>>(P, out);
-  } else {
-    if (lo) k_commit<T, 0, true><<<1216, 256, 0, s>>>(P, out);
-    else k_commit<T, 0, false><<<1216, 256, 0, s>>>(P, out);
+  const TileIdx ti = voxel_tiles(P.n);
+  const int nb = std::min(RBLOCKS, ti.ntile);
+#define FFTM_K(SL)                                                        \
+  if (tetra) {                                                            \
+    if (lo) k_commit<T, 1, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, out);  \
+    else k_commit<T, 1, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, out);    \
+  } else {                                                                \
+    if (lo) k_commit<T, 0, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, out);  \
+    else k_commit<T, 0, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, out);    \
   }
+  if (P.slaw == 1) { FFTM_K(1) } else if (P.slaw == 2) { FFTM_K(2) } else { FFTM_K(4) }
+#undef FFTM_K
   return cudaGetLastError();
 }
 
@@ -2054,13 +2077,18 @@ cudaError_t launch_state_io(const ResParams<T>& P, int tetra, T* out, const T* i
   return cudaGetLastError();
 }
 
-template <typename T, int TETRA, bool LO>
-__global__ void k_voxel_fields(ResParams<T> P, T* __restrict__ gout, T* __restrict__ sout) {
+template <typename T, int TETRA, bool LO, int SL>
+__global__ void __launch_bounds__(RTX * RTY) k_voxel_fields(ResParams<T> P, TileIdx ti, T* __restrict__ gout,
+                                                            T* __restrict__ sout) {
   const long long nv = (long long)P.n[0] * P.n[1] * P.n[2];
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv;
-       v += (long long)gridDim.x * blockDim.x) {
+  for (int t = blockIdx.x; t < ti.ntile; t += gridDim.x) {
+    int x0, y0, vz;
+    ti.at(t, &x0, &y0, &vz);
+    const int vx = x0 + (threadIdx.x % RTX), vy = y0 + (threadIdx.x / RTX);
+    if (vx >= P.n[0] || vy >= P.n[1]) continue;
+    const long long v = vx + vy * P.vy + (long long)vz * P.vz;
     T Gt[2][9], Pp[2][9];
-    voxel_eval<T, TETRA, LO>(P, v, Gt, Pp);
+    voxel_eval<T, TETRA, LO, SL>(P, vx, vy, vz, Gt, Pp);
 #pragma unroll
     for (int r = 0; r < (TETRA ? 2 : 1); ++r) {
       if (gout) {
@@ -2068,7 +2096,7 @@ __global__ void k_voxel_fields(ResParams<T> P, T* __restrict__ gout, T* __restri
         for (int i = 0; i < 9; ++i) gout[v + nv * (i + 9 * r)] = Gt[r][i];
       }
       if (sout && P.sym) {
-        const int map[6] = {0, 4, 8, 5, 2, 1};  // 11, 22, 33, 23, 13, 12
+        constexpr int map[6] = {0, 4, 8, 5, 2, 1};  // 11, 22, 33, 23, 13, 12
 #pragma unroll
         for (int c = 0; c < 6; ++c) sout[v + nv * (c + 6 * r)] = Pp[r][map[c]];
       } else if (sout) {
@@ -2082,51 +2110,143 @@ __global__ void k_voxel_fields(ResParams<T> P, T* __restrict__ gout, T* __restri
 template <typename T>
 cudaError_t launch_voxel_fields(const ResParams<T>& P, int tetra, T* grad_out, T* stress_out, cudaStream_t s) {
   const bool lo = P.ulo[0] != nullptr;
-  if (tetra) {
-    if (lo) k_voxel_fields<T, 1, true><<<1216, 256, 0, s>>>(P, grad_out, stress_out);
-    else k_voxel_fields<T, 1, false><<<1216, 256, 0, s>>>(P, grad_out, stress_out);
-  } else {
-    if (lo) k_voxel_fields<T, 0, true><<<1216, 256, 0, s>>>(P, grad_out, stress_out);
-    else k_voxel_fields<T, 0, false><<<1216, 256, 0, s>>>(P, grad_out, stress_out);
+  const TileIdx ti = voxel_tiles(P.n);
+  const int nb = std::min(RBLOCKS, ti.ntile);
+#define FFTM_K(SL)                                                                                     \
+  if (tetra) {                                                                                         \
+    if (lo) k_voxel_fields<T, 1, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, grad_out, stress_out);      \
+    else k_voxel_fields<T, 1, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, grad_out, stress_out);        \
+  } else {                                                                                             \
+    if (lo) k_voxel_fields<T, 0, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, grad_out, stress_out);      \
+    else k_voxel_fields<T, 0, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, grad_out, stress_out);        \
   }
+  FFTM_BY_LAW(P.slaw, FFTM_K);
+#undef FFTM_K
   return cudaGetLastError();
 }
 
-// ---- volume means of P and G (step report) ----
-template <typename T, int TETRA, bool LO>
-__global__ void __launch_bounds__(256) k_stats(ResParams<T> P, double* __restrict__ partial) {
-  __shared__ double red[32];
-  const long long nv = (long long)P.n[0] * P.n[1] * P.n[2];
-  double acc[18];
+// ---- volume means of P and G (step report, normal-mixed loading) ----
+// A sum of field values that keeps FP64's precision: FP64 adds for double data; for float data an
+// unevaluated pair of floats updated with TwoSum (this GPU's FP64 pipe takes a conversion or an
+// add of one warp every 16 cycles, so 18 sums in FP64 cost more than the law they sum).
+template <typename T>
+struct SumAcc {
+  T hi = T(0), lo = T(0);
+  __device__ __forceinline__ void add(T a) {
+    if constexpr (sizeof(T) == 8) {
+      hi += a;
+    } else {
+      const T s = hi + a, b = s - hi;
+      lo += (hi - (s - b)) + (a - b);
+      hi = s;
+    }
+  }
+  __device__ __forceinline__ double value() const { return sizeof(T) == 8 ? (double)hi : (double)hi + (double)lo; }
+};
+
+// Sums of NV accumulators over the block -> row[0 .. NV): one value per warp at a time from
+// shared memory, eight per lane and five shuffles (an eighth of the FP64 adds that shuffling
+// every warp's values takes).
+template <typename T, int NV>
+__device__ __forceinline__ void block_sums(const SumAcc<T> (&acc)[NV], double* __restrict__ row) {
+  constexpr int NT = RTX * RTY;
+  __shared__ double sm[NV][NT];
 #pragma unroll
-  for (int i = 0; i < 18; ++i) acc[i] = 0.0;
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv;
-       v += (long long)gridDim.x * blockDim.x) {
+  for (int i = 0; i < NV; ++i) sm[i][threadIdx.x] = acc[i].value();
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < NV; i += NT / 32) {
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < NT / 32; ++k) t += sm[i][lane + 32 * k];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (lane == 0) row[i] = t;
+  }
+}
+
+template <typename T, int TETRA, bool LO, int SL>
+__global__ void __launch_bounds__(RTX * RTY) k_stats(ResParams<T> P, TileIdx ti, double* __restrict__ partial) {
+  SumAcc<T> acc[18];
+  for (int t = blockIdx.x; t < ti.ntile; t += gridDim.x) {
+    int x0, y0, vz;
+    ti.at(t, &x0, &y0, &vz);
+    const int vx = x0 + (threadIdx.x % RTX), vy = y0 + (threadIdx.x / RTX);
+    if (vx >= P.n[0] || vy >= P.n[1]) continue;
     T Gt[2][9], Pp[2][9];
-    voxel_eval<T, TETRA, LO>(P, v, Gt, Pp);
+    voxel_eval<T, TETRA, LO, SL>(P, vx, vy, vz, Gt, Pp);
 #pragma unroll
     for (int r = 0; r < (TETRA ? 2 : 1); ++r)
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
-        acc[i] += (double)Pp[r][i];
-        acc[9 + i] += (double)Gt[r][i];
+        acc[i].add(Pp[r][i]);
+        acc[9 + i].add(Gt[r][i]);
       }
   }
-  for (int i = 0; i < 18; ++i) {
-    const double t = block_sum(acc[i], red);
-    if (threadIdx.x == 0) partial[(size_t)blockIdx.x * 18 + i] = t;
+  block_sums<T, 18>(acc, partial + (size_t)blockIdx.x * 18);
+}
+
+constexpr int STATS_BLOCKS = 152 * 4;  // rows of partials at most (each block ends with 18 FP64 sums)
+
+template <typename T>
+cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s) {
+  const bool lo = P.ulo[0] != nullptr;
+  const TileIdx ti = voxel_tiles(P.n);
+  const int nb = std::min(STATS_BLOCKS, ti.ntile);
+  *nblocks = nb;
+#define FFTM_K(SL)                                                                     \
+  if (tetra) {                                                                         \
+    if (lo) k_stats<T, 1, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, partial);          \
+    else k_stats<T, 1, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, partial);            \
+  } else {                                                                             \
+    if (lo) k_stats<T, 0, true, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, partial);          \
+    else k_stats<T, 0, false, SL><<<nb, RTX * RTY, 0, s>>>(P, ti, partial);            \
   }
+  FFTM_BY_LAW(P.slaw, FFTM_K);
+#undef FFTM_K
+  return cudaGetLastError();
+}
+
+// The sum of P alone, from the voxel-point stresses that the two-pass residual has just stored
+// (its plain form): normal-mixed loading needs the mean stress after every residual, and
+// evaluating every point's law again for it cost as much as the residual's own k_stress
+// (103 us an iteration of a 64^3 FP64 problem).
+template <typename T, int NPP, bool SYM>
+__global__ void __launch_bounds__(RTX * RTY) k_stress_sums(const T* __restrict__ vs, long long nvox,
+                                                           double* __restrict__ partial) {
+  constexpr int NC = SYM ? 6 : 9;
+  SumAcc<T> acc[9];
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox;
+       v += (long long)gridDim.x * blockDim.x) {
+    T p[NPP][NC];
+#pragma unroll
+    for (int r = 0; r < NPP; ++r)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) p[r][c] = __ldg(vs + (size_t)(r * NC + c) * nvox + v);
+#pragma unroll
+    for (int r = 0; r < NPP; ++r)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c].add(p[r][c]);
+  }
+  if (SYM) {  // (11, 22, 33, 23, 13, 12) -> P[3 i + q]
+    const SumAcc<T> a0 = acc[0], a1 = acc[1], a2 = acc[2], a3 = acc[3], a4 = acc[4], a5 = acc[5];
+    acc[0] = a0; acc[1] = a5; acc[2] = a4;
+    acc[3] = a5; acc[4] = a1; acc[5] = a3;
+    acc[6] = a4; acc[7] = a3; acc[8] = a2;
+  }
+  block_sums<T, 9>(acc, partial + (size_t)blockIdx.x * 9);
 }
 
 template <typename T>
-cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int nblocks, cudaStream_t s) {
-  const bool lo = P.ulo[0] != nullptr;
+cudaError_t launch_stress_sums(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s) {
+  const long long nvox = (long long)P.n[0] * P.n[1] * P.n[2];
+  const int nb = (int)std::min<long long>(STATS_BLOCKS, (nvox + RTX * RTY - 1) / (RTX * RTY));
+  *nblocks = nb;
   if (tetra) {
-    if (lo) k_stats<T, 1, true><<<nblocks, 256, 0, s>>>(P, partial);
-    else k_stats<T, 1, false><<<nblocks, 256, 0, s>>>(P, partial);
+    if (P.sym) k_stress_sums<T, 2, true><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
+    else k_stress_sums<T, 2, false><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
   } else {
-    if (lo) k_stats<T, 0, true><<<nblocks, 256, 0, s>>>(P, partial);
-    else k_stats<T, 0, false><<<nblocks, 256, 0, s>>>(P, partial);
+    if (P.sym) k_stress_sums<T, 1, true><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
+    else k_stress_sums<T, 1, false><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
   }
   return cudaGetLastError();
 }
