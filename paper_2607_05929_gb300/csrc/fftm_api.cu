@@ -86,47 +86,86 @@ double kind_xi(int kind, int n, int k, bool* zero, bool* pi) {
   }
 }
 
-bool factor_radices(int M, std::vector<int>* rad) {
-  rad->clear();
-  int m = M;
-  while (m % 3 == 0) { rad->push_back(3); m /= 3; }
-  while (m % 8 == 0) { rad->push_back(8); m /= 8; }
-  while (m % 4 == 0) { rad->push_back(4); m /= 4; }
-  while (m % 2 == 0) { rad->push_back(2); m /= 2; }
-  return m == 1 && (int)rad->size() <= MAX_STAGES;
+bool smooth23(int m) {
+  while (m % 3 == 0) m /= 3;
+  while (m % 2 == 0) m /= 2;
+  return m == 1;
+}
+
+// N as a product of exactly S of the radices the passes have, with the smallest sum (balanced
+// stages); false if there is none.
+bool factor_stages(int N, int S, int* rad) {
+  static const int kRadix[] = {16, 12, 9, 8, 6, 4, 3, 2};
+  if (S == 1) {
+    for (int r : kRadix)
+      if (r == N) {
+        rad[0] = r;
+        return true;
+      }
+    return false;
+  }
+  int best = 0;
+  for (int r : kRadix) {
+    int rest[MAX_STAGES];
+    if (N % r != 0 || !factor_stages(N / r, S - 1, rest)) continue;
+    int sum = r;
+    for (int s = 0; s + 1 < S; ++s) sum += rest[s];
+    if (best && sum >= best) continue;
+    best = sum;
+    rad[0] = r;
+    for (int s = 0; s + 1 < S; ++s) rad[s + 1] = rest[s];
+  }
+  return best > 0;
 }
 
 struct HostPlan {
-  int kind, n, lo, L, M;
-  std::vector<int> radix;
-  std::vector<int16_t> perm;
+  int kind, n, lo, L;
+  int lev, nseg, nst, total;
+  SegPlan seg[MAX_SEGS];
   std::vector<double> tw;  // interleaved re, im
   std::vector<double> qw;
 };
 
+// A type-I transform splits twice from 16 voxels up, once from 8, where n has the factors of two:
+// below, the halves are too short to gain anything.
 HostPlan make_plan(int kind, int n) {
   HostPlan p;
   p.kind = kind;
   p.n = n;
   kind_range(kind, n, &p.lo, &p.L);
-  p.M = (kind == K_DFT) ? n : 2 * n;
-  factor_radices(p.M, &p.radix);
-  const int S = (int)p.radix.size();
-  std::vector<int> Lw(S + 1, 1);  // Lw[s] = R_0 ... R_{s-1}
-  for (int s = 0; s < S; ++s) Lw[s + 1] = Lw[s] * p.radix[s];
-  p.perm.resize(p.M);
-  for (int j = 0; j < p.M; ++j) {
-    int rem = j, pos = 0;
-    for (int s = S - 1; s >= 0; --s) {
-      const int r = rem % p.radix[s];
-      rem /= p.radix[s];
-      pos += r * Lw[s];
-    }
-    p.perm[j] = (int16_t)pos;
+  std::memset(p.seg, 0, sizeof(p.seg));
+  const bool type1 = kind == K_DCT1 || kind == K_DST1;
+  p.lev = !type1 ? 0 : (n >= 16 && n % 4 == 0) ? 2 : (n >= 8 && n % 2 == 0) ? 1 : 0;
+  p.nseg = p.lev + 1;
+  p.total = 0;
+  int ntab = 0;
+  for (int g = 0; g < p.nseg; ++g) {
+    SegPlan& sg = p.seg[g];
+    const bool last = g == p.lev;
+    sg.N = !type1 ? n : last ? 2 * (n >> p.lev) : n >> (g + 1);
+    sg.off = p.total;
+    p.total += sg.N;
+    ntab = std::max(ntab, sg.N);
   }
-  p.tw.resize(2 * p.M);
-  for (int t = 0; t < p.M; ++t) {
-    const double a = -2.0 * kPi * t / p.M;
+  for (p.nst = 1; p.nst <= MAX_STAGES; ++p.nst) {  // the fewest stages that every segment can take
+    bool ok = true;
+    for (int g = 0; g < p.nseg; ++g) ok = ok && factor_stages(p.seg[g].N, p.nst, p.seg[g].rad);
+    if (ok) break;
+  }
+  for (int g = 0; g < p.nseg; ++g) {
+    SegPlan& sg = p.seg[g];
+    int lp = 1;
+    for (int s = 0; s < p.nst && s < MAX_STAGES; ++s) {
+      sg.nb[s] = sg.N / sg.rad[s];
+      sg.lp[s] = lp;
+      sg.tstep[s] = ntab / (lp * sg.rad[s]);
+      sg.magic[s] = lp > 1 ? (unsigned)((0x100000000ull + lp - 1) / lp) : 0u;
+      lp *= sg.rad[s];
+    }
+  }
+  p.tw.resize(2 * (size_t)ntab);
+  for (int t = 0; t < ntab; ++t) {
+    const double a = -2.0 * kPi * t / ntab;
     p.tw[2 * t] = std::cos(a);
     p.tw[2 * t + 1] = std::sin(a);
   }
@@ -315,8 +354,7 @@ struct fftm_problem {
   size_t off_tcxf[3][3], off_tcxi[3][3];  // TF32 y, z with 257 outputs: output 256's row
   int tcx[3][3];
   // device table offsets (bytes) inside `tables`
-  size_t off_perm[3][3], off_tw[3][3], off_qw[3][3], off_S2[3][3], off_C2[3][3];
-  int maxM[3], maxL[3];
+  size_t off_tw[3][3], off_qw[3][3], off_S2[3][3], off_C2[3][3];
   int cur = 0;  // ring slot holding the current u^f
   int res_passes = 0;     // requested residual form: 0 tuned, 1 one pass, 2 two passes
   int res_two_pass = -1;  // resolved form (-1: not yet)
@@ -446,10 +484,11 @@ AxisPlan<T> dev_plan(fftm_problem* p, int q, int a) {
   d.n = h.n;
   d.lo = h.lo;
   d.L = h.L;
-  d.M = h.M;
-  d.nst = (int)h.radix.size();
-  for (int s = 0; s < MAX_STAGES; ++s) d.radix[s] = s < d.nst ? h.radix[s] : 1;
-  d.perm = reinterpret_cast<const int16_t*>(reinterpret_cast<char*>(p->tables) + p->off_perm[q][a]);
+  d.lev = h.lev;
+  d.nseg = h.nseg;
+  d.nst = h.nst;
+  d.total = h.total;
+  for (int g = 0; g < MAX_SEGS; ++g) d.seg[g] = h.seg[g];
   d.tw = tptr_v2<T>(p, p->off_tw[q][a]);
   d.qw = tptr_v2<T>(p, p->off_qw[q][a]);
   return d;
@@ -497,7 +536,7 @@ PassParams<T> pass_params(fftm_problem* p, int axis, int inverse, int fused, int
 template <typename T>
 int launch_pp(fftm_problem* p, const PassParams<T>& P, int axis) {
   ProfScope ps(p, axis == 0 ? FFTM_KCAT_PASS_X : (axis == 1 ? FFTM_KCAT_PASS_Y : FFTM_KCAT_PASS_Z));
-  CU(launch_pass<T>(P, p->maxM[axis], p->maxL[axis], p->n[axis], p->ctx->stream));
+  CU(launch_pass<T>(P, p->ctx->stream));
   p->launches++;
   return FFTM_OK;
 }
@@ -1557,8 +1596,7 @@ int validate(const fftm_problem_desc* d) {
   for (int a = 0; a < 3; ++a) {
     const bool per = d->bc[a][0][0] == FFTM_BC_PERIODIC;
     const int M = per ? d->n[a] : 2 * d->n[a];
-    std::vector<int> r;
-    if (!factor_radices(M, &r)) return set_err(FFTM_E_UNSUPPORTED, "grid sizes must be 2^a 3^b");
+    if (!smooth23(M)) return set_err(FFTM_E_UNSUPPORTED, "grid sizes must be 2^a 3^b");
     if (M > 2048) return set_err(FFTM_E_UNSUPPORTED, "transform length above 2048");
   }
   return FFTM_OK;
@@ -1794,14 +1832,6 @@ static int problem_create(fftm_ctx* ctx, const fftm_problem_desc* desc0, void* w
       p->hi[q][a] = lo + L;
       p->plans[q][a] = make_plan(p->kind[q][a], p->n[a]);
     }
-  for (int a = 0; a < 3; ++a) {
-    p->maxM[a] = 0;
-    p->maxL[a] = 0;
-    for (int q = 0; q < 3; ++q) {
-      p->maxM[a] = std::max(p->maxM[a], p->plans[q][a].M);
-      p->maxL[a] = std::max(p->maxL[a], p->plans[q][a].L);
-    }
-  }
   // ---- device allocations ----
   const cudaStream_t s = ctx->stream;
   if (dev_alloc(p.get(), reinterpret_cast<void**>(&p->fields), sz.fields) != cudaSuccess) {
@@ -1858,7 +1888,6 @@ static int problem_create(fftm_ctx* ctx, const fftm_problem_desc* desc0, void* w
   for (int q = 0; q < 3; ++q)
     for (int a = 0; a < 3; ++a) {
       const HostPlan& h = p->plans[q][a];
-      p->off_perm[q][a] = put(h.perm.data(), h.perm.size() * sizeof(int16_t));
       std::vector<double> s2(h.L), c2(h.L);
       for (int k = 0; k < h.L; ++k) {
         bool z, pi;

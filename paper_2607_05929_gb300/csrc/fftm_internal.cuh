@@ -17,21 +17,29 @@ template <typename T> struct V2;
 template <> struct V2<float> { using t = float2; };
 template <> struct V2<double> { using t = double2; };
 
-constexpr int MAX_STAGES = 16;
+constexpr int MAX_STAGES = 4, MAX_SEGS = 3;
 
-// Plan of the 1D transform of one displacement component along one axis.
-// Every DT is evaluated through one complex FFT of length M (M = n for the
-// DFT, 2n for the DCT/DST kinds), two real pencils packed per complex pencil.
+// One complex FFT of a transform's plan: length N at rows off of the work buffer, its Stockham
+// stages (radix, butterflies N / R, product Lp of the radices before, ceil(2^32 / Lp), twiddle
+// step ntab / (Lp R)).
+struct SegPlan {
+  int N, off;
+  int rad[MAX_STAGES], nb[MAX_STAGES], lp[MAX_STAGES], tstep[MAX_STAGES];
+  unsigned magic[MAX_STAGES];
+};
+
+// Plan of the 1D transform of one displacement component along one axis (fftm_dt.cu): type-I
+// transforms split lev times, the FFTs of two real pencils packed per complex pencil, the same
+// number of stages in every segment.
 template <typename T>
 struct AxisPlan {
   int kind;
   int n;      // voxels along the axis
   int lo, L;  // node range of the transform (positions lo .. lo + L - 1)
-  int M;      // complex FFT length
-  int nst;    // number of FFT stages
-  int radix[MAX_STAGES];
-  const int16_t* perm;               // M: input position of sequence index m
-  const typename V2<T>::t* tw;       // M: exp(-2 pi i t / M)
+  int lev, nseg, nst;
+  int total;                         // rows of the work buffer: sum of the segment lengths
+  SegPlan seg[MAX_SEGS];
+  const typename V2<T>::t* tw;       // ntab (the longest segment): exp(-2 pi i t / ntab)
   const typename V2<T>::t* qw;       // n + 1: exp(i pi j / (2 n))
 };
 
@@ -251,7 +259,7 @@ struct C0Params {
 
 // ---- launchers (return cudaError_t of the launch) ----
 template <typename T>
-cudaError_t launch_pass(const PassParams<T>& P, int maxM, int maxL, int maxn, cudaStream_t s);
+cudaError_t launch_pass(const PassParams<T>& P, cudaStream_t s);
 template <typename T>
 cudaError_t launch_green_c0(const C0Params<T>& P, cudaStream_t s);
 template <typename T>
