@@ -310,8 +310,9 @@ struct fftm_problem {
   void* tables = nullptr;  // plans + green tables
   uint16_t* phase = nullptr;
   int* law_id = nullptr;
+  int one_law = -1;  // the law that every phase has, if they share one
   void* law_c = nullptr;
-  void* law_m = nullptr;  // elastic phases: the 6x6 Mandel stiffness in (2 x 2)-pair order, 36 per phase
+  void* law_m = nullptr;  // elastic phases: the 6x6 stiffness in (2 x 2)-pair order, 36 per phase
   double* partial = nullptr;
   size_t partial_len = 0;
   double* dscal = nullptr;  // [0..1] norms, [2..9] anderson coef, [16..] stats
@@ -660,6 +661,7 @@ ResParams<T> res_params(fftm_problem* p, int slot, T* D_base, T* p_base) {
   }
   R.phase = p->phase;
   R.law_id = p->law_id;
+  R.one_law = p->one_law;
   R.law_c = reinterpret_cast<const T*>(p->law_c);
   R.law_m = reinterpret_cast<const T*>(p->law_m);
   for (int a = 0; a < 3; ++a) {
@@ -677,6 +679,13 @@ ResParams<T> res_params(fftm_problem* p, int slot, T* D_base, T* p_base) {
   R.vz = (long long)p->n[0] * p->n[1];
   for (int i = 0; i < 3; ++i)
     for (int q = 0; q < 3; ++q) R.Gs[i * 3 + q] = T(p->load.A[q][i]);  // G*_iq = d u*_q / d x_i
+  for (int k = 0; k < 6; ++k) {  // 11, 22, 33, 23, 13, 12
+    static const int ij[6][2] = {{0, 0}, {1, 1}, {2, 2}, {1, 2}, {0, 2}, {0, 1}};
+    const int i = ij[k][0], j = ij[k][1];
+    auto strain = [&](const double (&A)[3][3]) { return k < 3 ? A[i][i] : A[i][j] + A[j][i]; };
+    R.e0[k] = T(strain(p->load.A));
+    R.de0[k] = T(strain(p->load.A) - strain(p->load_n.A));
+  }
   const double lam0 = p->desc.green == FFTM_GREEN_MU0 ? 0.0 : p->desc.lambda0;
   R.lam0 = T(lam0);
   R.two_mu0 = T(2.0 * p->desc.mu0);
@@ -2017,6 +2026,7 @@ static int problem_create(fftm_ctx* ctx, const fftm_problem_desc* desc0, void* w
   for (int i = 0; i < desc->n_phases; ++i) {
     const fftm_material& m = desc->materials[i];
     lid[i] = m.law;
+    p->one_law = i == 0 || p->one_law == m.law ? m.law : -1;
     double* c = &lc[(size_t)i * LAWC];
     if (m.law == FFTM_LAW_CUBIC_ELASTIC || m.law == FFTM_LAW_SVK_CUBIC) {
       double R[3][3], Cm[6][6];
@@ -2044,8 +2054,9 @@ static int problem_create(fftm_ctx* ctx, const fftm_problem_desc* desc0, void* w
       c[1] = m.params[1];
     }
   }
-  // the small-strain elastic phases' Mandel stiffness for the one-pass residual: float4 k = 3 bp + rp
-  // holds (C[2rp][2bp], C[2rp+1][2bp], C[2rp][2bp+1], C[2rp+1][2bp+1]) (isotropic: lambda 1 (x) 1 + 2 mu I)
+  // the small-strain elastic phases' stiffness for the residual, from strains with engineering shears
+  // to stresses (the Mandel one with its shear rows and columns over sqrt 2; isotropic: lambda 1 (x) 1
+  // + 2 mu I): block k = 3 bp + rp holds C[2rp][2bp], C[2rp+1][2bp], C[2rp][2bp+1], C[2rp+1][2bp+1]
   std::vector<double> lm((size_t)desc->n_phases * 36, 0.0);
   for (int i = 0; i < desc->n_phases; ++i) {
     const fftm_material& m = desc->materials[i];
@@ -2059,6 +2070,10 @@ static int problem_create(fftm_ctx* ctx, const fftm_problem_desc* desc0, void* w
         for (int b = 0; b < 3; ++b) Cm[a][b] = m.params[0];
       for (int a = 0; a < 6; ++a) Cm[a][a] += 2.0 * m.params[1];
     }
+    for (int a = 0; a < 6; ++a)
+      for (int b = 0; b < 6; ++b)
+        if ((a < 3) != (b < 3)) Cm[a][b] *= std::sqrt(0.5);
+        else if (a >= 3) Cm[a][b] *= 0.5;
     double* c = &lm[(size_t)i * 36];
     for (int bp = 0; bp < 3; ++bp)
       for (int rp = 0; rp < 3; ++rp) {

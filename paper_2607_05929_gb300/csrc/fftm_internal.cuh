@@ -81,8 +81,9 @@ struct ResParams {
   T* p[3];          // p = div(R0 : grad u^f) - D (test variant only)
   const uint16_t* phase;
   const int* law_id;  // per phase
+  int one_law;        // the law of every phase, or -1: a kernel-wide value needs no load
   const T* law_c;     // per phase, LAWC coefficients
-  const T* law_m;     // per phase, the elastic Mandel stiffness as 9 (2 x 2) blocks (36 entries)
+  const T* law_m;     // per phase, the elastic stiffness as 9 (2 x 2) blocks (36 entries)
   int n[3], N[3];
   int periodic[3];
   long long sy, sz;  // node strides (x stride 1)
@@ -116,6 +117,7 @@ struct ResParams {
   T lam0, two_mu0;
   T wdiv[3];         // 1 / (4 h_i)
   T wgrad[3];        // HEX1: 1 / (4 h_i); TETRA2: 1 / (2 h_i)
+  T e0[6], de0[6];   // strains (engineering shears) of Gs and dGs
   int sgn[3][3][2];  // [q][axis][face] +1 symmetric (Neumann), -1 anti-symmetric (Dirichlet)
   int lo[3][3], hi[3][3];  // [q][axis] transformed node range
   // Uniform Neumann tractions tr[axis][face][q] (outward normal convention); at the nodes of

@@ -571,12 +571,11 @@ __device__ __forceinline__ void law_eval(int law, const T* __restrict__ c, const
 // this way every rounding is relative to the increment, not to the stress.
 // c = (lambda, mu, sigma_y, H).  dP (may be null): P - P_n; Pf: P; stn (may be
 // null): the returned state (e_{n+1} = volumetric part + k times the deviator).
+// j2_strain: on the strain increment de, stresses as (11, 22, 33, 23, 13, 12); j2_inc: on dG.
 template <typename T>
-__device__ __forceinline__ void j2_inc(const T* __restrict__ c, const T dG[9], const T st[7], T* dP, T Pf[9],
-                                       T* stn) {
+__device__ __forceinline__ void j2_strain(const T* __restrict__ c, const T de[6], const T st[7], T d6[6], T p6[6],
+                                          T* stn) {
   const T lam = __ldg(c), mu = __ldg(c + 1), sy = __ldg(c + 2), H = __ldg(c + 3);
-  const T de[6] = {dG[0], dG[4], dG[8], T(0.5) * (dG[5] + dG[7]), T(0.5) * (dG[2] + dG[6]),
-                   T(0.5) * (dG[1] + dG[3])};
   const T dtr = de[0] + de[1] + de[2], dm = dtr * T(1.0 / 3.0);
   const T trn = st[0] + st[1] + st[2], mn = trn * T(1.0 / 3.0);
   const T dd[6] = {de[0] - dm, de[1] - dm, de[2] - dm, de[3], de[4], de[5]};
@@ -597,22 +596,30 @@ __device__ __forceinline__ void j2_inc(const T* __restrict__ c, const T dG[9], c
     km1 = -T(3) * mu * dp / q;
   }
   const T K = lam + T(2.0 / 3.0) * mu, m2 = T(2) * mu;
-  T d6[6], p6[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     d6[i] = m2 * ((T(1) + km1) * dd[i] + km1 * dn[i]) + (i < 3 ? K * dtr : T(0));
     p6[i] = (m2 * dn[i] + (i < 3 ? K * trn : T(0))) + d6[i];
   }
+  if (stn) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) stn[i] = (i < 3 ? mn + dm : T(0)) + (T(1) + km1) * (dn[i] + dd[i]);
+    stn[6] = st[6] + dp;
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void j2_inc(const T* __restrict__ c, const T dG[9], const T st[7], T* dP, T Pf[9],
+                                       T* stn) {
+  const T de[6] = {dG[0], dG[4], dG[8], T(0.5) * (dG[5] + dG[7]), T(0.5) * (dG[2] + dG[6]),
+                   T(0.5) * (dG[1] + dG[3])};
+  T d6[6], p6[6];
+  j2_strain<T>(c, de, st, d6, p6, stn);
   constexpr int map9[9] = {0, 5, 4, 5, 1, 3, 4, 3, 2};  // G[i*3+q] -> symmetric slot
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     Pf[i] = p6[map9[i]];
     if (dP) dP[i] = d6[map9[i]];
-  }
-  if (stn) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) stn[i] = (i < 3 ? mn + dm : T(0)) + (T(1) + km1) * (dn[i] + dd[i]);
-    stn[6] = st[6] + dp;
   }
 }
 
@@ -726,6 +733,179 @@ __device__ __forceinline__ void law_grad(const ResParams<T>& P, bool j2, const T
   }
 }
 
+// ---- small-strain laws straight from the stencil sums ------------------------------------
+// The differences of one displacement component along the three axes at a voxel point, from its
+// corner values (corner o = ox + 2 oy + 4 oz; sub and add in the field's arithmetic, packed
+// (hi, lo) pairs in FP32): the four-term sums of point_grad share their parts -- HEX1: the four
+// body diagonals' differences a, b, c, d give x = (a + b) + (c - d), y = (a + b) - (c - d),
+// z = (a - b) + (c + d), 11 operations for the three axes instead of 24; TETRA2: the tetrahedron's
+// four corners give x = A + B, y = A - B and z in 7 instead of 12.  Every term is still a
+// difference of neighbouring values.
+// The FP64 residual is bound by the FP64 pipe (two FMA a clock and SM), so these sums, the strain
+// and the divergence below in fewer operations are its time: 128^3 TETRA2 k_stress 778 -> 565 us,
+// k_div 355 -> 230 us.  FP32 issues fewer instructions (one pass, 192^3: 239 -> 226 us; 256^3 with
+// low parts 601 -> 519 us).
+struct ScalarOps {
+  template <typename V> static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
+  template <typename V> static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+};
+struct PairOps {  // FP32 (hi, lo), packed FP32x2 instructions
+  static __device__ __forceinline__ float2 sub(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+  }
+  static __device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+};
+
+template <typename Ops, int TETRA, typename V, typename U>
+__device__ __forceinline__ void corner_diffs(U&& u, int r, V s[3]) {
+  if constexpr (TETRA) {
+    // T1: corners 0 (000), 3 (110), 5 (101), 6 (011); T2: their opposites, whose differences along
+    // each axis are those of the point reflection
+    const V p = u(r == 0 ? 3 : 4), o = u(r == 0 ? 0 : 7), m = u(r == 0 ? 5 : 2), n = u(r == 0 ? 6 : 1);
+    const V A = r == 0 ? Ops::sub(p, o) : Ops::sub(o, p), B = r == 0 ? Ops::sub(m, n) : Ops::sub(n, m);
+    s[0] = Ops::add(A, B);
+    s[1] = Ops::sub(A, B);
+    s[2] = r == 0 ? Ops::add(Ops::sub(m, o), Ops::sub(n, p)) : Ops::add(Ops::sub(o, m), Ops::sub(p, n));
+  } else {
+    const V a = Ops::sub(u(7), u(0)), b = Ops::sub(u(3), u(4)), c = Ops::sub(u(5), u(2)), d = Ops::sub(u(6), u(1));
+    const V ab = Ops::add(a, b), cd = Ops::sub(c, d);
+    s[0] = Ops::add(ab, cd);
+    s[1] = Ops::sub(ab, cd);
+    s[2] = Ops::add(Ops::sub(a, b), Ops::add(c, d));
+  }
+}
+
+// Strain (11, 22, 33, and the engineering shears 23, 13, 12) from the sums s[q][i] of component q
+// along axis i: the weights, the symmetric part and the affine load's strain (e0) in one FMA per
+// sum, and no factor of sqrt 2 to round.
+// (FMAs are spelled out here and below: the one-pass and the two-pass residual then round alike,
+// whatever the compiler contracts in either kernel, and give the same iterates.)
+template <typename T>
+__device__ __forceinline__ void sum_strain(const T s[3][3], const T* w, const T* e0, T e[6]) {
+  e[0] = fma(w[0], s[0][0], e0[0]);
+  e[1] = fma(w[1], s[1][1], e0[1]);
+  e[2] = fma(w[2], s[2][2], e0[2]);
+  e[3] = fma(w[1], s[2][1], fma(w[2], s[1][2], e0[3]));
+  e[4] = fma(w[0], s[2][0], fma(w[2], s[0][2], e0[4]));
+  e[5] = fma(w[0], s[1][0], fma(w[1], s[0][1], e0[5]));
+}
+
+// The strain of the quadratic part of u* (add_quad) added to e.
+template <typename T, int TETRA>
+__device__ __forceinline__ void add_quad_strain(const T hh[3], const T Q[3][6], int r, int vx, int vy, int vz,
+                                                T e[6]) {
+  T G[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  add_quad<T, TETRA>(hh, Q, r, vx, vy, vz, G);
+  e[0] += G[0];
+  e[1] += G[4];
+  e[2] += G[8];
+  e[3] += G[5] + G[7];
+  e[4] += G[2] + G[6];
+  e[5] += G[1] + G[3];
+}
+
+// Cubic elasticity on the strain e: stresses p (11, 22, 33, 23, 13, 12) with the phase's stiffness
+// m36 (ResParams::law_m).  FP32: packed products of all 36 entries; FP64: the upper triangle's six
+// 2 x 2 blocks.
+__device__ __forceinline__ void cubic_strain(const float* __restrict__ m36, const float e[6], float p[6]) {
+  const float4* M4 = reinterpret_cast<const float4*>(m36);
+  float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int bp = 0; bp < 3; ++bp) {
+    const float2 e0 = make_float2(e[2 * bp], e[2 * bp]), e1 = make_float2(e[2 * bp + 1], e[2 * bp + 1]);
+#pragma unroll
+    for (int rp = 0; rp < 3; ++rp) {
+      const float4 c = __ldg(M4 + 3 * bp + rp);
+      acc[rp] = __ffma2_rn(make_float2(c.x, c.y), e0, acc[rp]);
+      acc[rp] = __ffma2_rn(make_float2(c.z, c.w), e1, acc[rp]);
+    }
+  }
+#pragma unroll
+  for (int rp = 0; rp < 3; ++rp) {
+    p[2 * rp] = acc[rp].x;
+    p[2 * rp + 1] = acc[rp].y;
+  }
+}
+__device__ __forceinline__ void cubic_strain(const double* __restrict__ m36, const double e[6], double p[6]) {
+  const double2* M2 = reinterpret_cast<const double2*>(m36);
+  double C[6][6];
+#pragma unroll
+  for (int bp = 0; bp < 3; ++bp)
+#pragma unroll
+    for (int rp = 0; rp <= bp; ++rp) {
+      const double2 a = __ldg(M2 + 2 * (3 * bp + rp)), b = __ldg(M2 + 2 * (3 * bp + rp) + 1);
+      C[2 * rp][2 * bp] = a.x;
+      C[2 * rp + 1][2 * bp] = a.y;
+      C[2 * rp][2 * bp + 1] = b.x;
+      C[2 * rp + 1][2 * bp + 1] = b.y;
+    }
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    double t = C[0][a] * e[0];
+#pragma unroll
+    for (int b = 1; b < 6; ++b) t = fma(a < b ? C[a][b] : C[b][a], e[b], t);
+    p[a] = t;
+  }
+}
+
+// Small-strain elastic law of a phase at NP points (c: its law row; an isotropic phase keeps its
+// two constants, fewer products and roundings than the full stiffness).  One branch for the points
+// together: their products interleave and the stiffness is loaded once (the 192^3 FP32 one-pass
+// residual: 232 us, 248 with a branch per point).
+template <typename T, int NP>
+__device__ __forceinline__ void elastic_strain(int law, const T* __restrict__ c, const T* __restrict__ m36,
+                                               const T (&e)[NP][6], T (&p)[NP][6]) {
+  if (law == LAW_CUBIC) {
+#pragma unroll
+    for (int r = 0; r < NP; ++r) cubic_strain(m36, e[r], p[r]);
+  } else {
+    const T lam = __ldg(c), mu = __ldg(c + 1), mu2 = T(2) * mu;
+#pragma unroll
+    for (int r = 0; r < NP; ++r) {
+      const T tr = lam * ((e[r][0] + e[r][1]) + e[r][2]);
+#pragma unroll
+      for (int a = 0; a < 6; ++a) p[r][a] = a < 3 ? fma(mu2, e[r][a], tr) : mu * e[r][a];
+    }
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ T (&one(T (&a)[6]))[1][6] { return *reinterpret_cast<T(*)[1][6]>(&a); }
+
+template <typename T>
+__device__ __forceinline__ T norm6(const T p[6]) {  // |P|^2
+  return fma(T(2), fma(p[3], p[3], fma(p[4], p[4], p[5] * p[5])), fma(p[0], p[0], fma(p[1], p[1], p[2] * p[2])));
+}
+
+// Node divergence of a symmetric stress, v(c, o) its component c (11, 22, 33, 23, 13, 12) at the
+// voxel point on corner o: the sums over the corners along axis i, sum over pairs of differences.
+// A shear component is differenced along two axes i, j: the differences along the face diagonals,
+// A = sum (v_11 - v_00) and B = sum (v_10 - v_01), give A + B and A - B: 54 operations for the
+// three components of D instead of 81.
+template <typename T, typename V>
+__device__ __forceinline__ void sym_div(V&& v, const T* w, T D[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int lowbits = (1 << i) - 1, o = ((k & ~lowbits) << 1) | (k & lowbits);  // corners with o_i = 0
+      const T d = v(i, o | (1 << i)) - v(i, o);
+      s = k == 0 ? d : s + d;
+    }
+    D[i] = w[i] * s;
+  }
+#pragma unroll
+  for (int c = 3; c < 6; ++c) {
+    const int i = c == 3 ? 1 : 0, j = c == 5 ? 1 : 2, m = 3 - i - j;  // the two axes, and the third
+    const int bi = 1 << i, bj = 1 << j, bm = 1 << m;
+    const T A = (v(c, bi | bj) - v(c, 0)) + (v(c, bi | bj | bm) - v(c, bm));
+    const T B = (v(c, bi) - v(c, bj)) + (v(c, bi | bm) - v(c, bj | bm));
+    D[j] = fma(w[i], A + B, D[j]);
+    D[i] = fma(w[j], A - B, D[i]);
+  }
+}
+
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -808,8 +988,71 @@ __device__ __forceinline__ int sym_index(int i, int q) {
   return 6 - i - q;  // (1,2) -> 3, (0,2) -> 4, (0,1) -> 5
 }
 
+// The sums s[q][i] of corner_diffs at point r from the corner values uh (+ ul with LO).
+template <typename T, int TETRA, bool LO>
+__device__ __forceinline__ void point_sums(const T uh[3][8], const T ul[3][8], int r, T s[3][3]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if constexpr (LO) {
+      float2 t[3];
+      corner_diffs<PairOps, TETRA, float2>([&](int o) { return make_float2(uh[q][o], ul[q][o]); }, r, t);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) s[q][i] = t[i].x + t[i].y;
+    } else {
+      corner_diffs<ScalarOps, TETRA, T>([&](int o) { return uh[q][o]; }, r, s[q]);
+    }
+  }
+}
+
+// The stresses of one voxel for the laws of a SYM problem (isotropic, cubic, J2), stored at its
+// points; |P|^2 added to *spv.  uh, ul: the corner values, less u^f_n in a J2 voxel.
+template <typename T, int TETRA, bool LO, bool J2>
+__device__ __forceinline__ void stress_sym(const ResParams<T>& P, int law, const T* __restrict__ lc,
+                                           const T* __restrict__ lm, bool j2,
+                                           const T uh[3][8], const T ul[3][8], int vx, int vy, int vz, int v,
+                                           long long nvox, T* spv) {
+#pragma unroll
+  for (int r = 0; r < (TETRA ? 2 : 1); ++r) {
+    T s[3][3], em[6], p6[6];
+    point_sums<T, TETRA, LO>(uh, ul, r, s);
+    T e0[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) e0[c] = (J2 && j2) ? P.de0[c] : P.e0[c];
+    sum_strain<T>(s, P.wgrad, e0, em);
+    if (J2 && j2) {
+      if (P.dquad) add_quad_strain<T, TETRA>(P.hh, P.dQ, r, vx, vy, vz, em);
+    } else if (P.quad) {
+      add_quad_strain<T, TETRA>(P.hh, P.Qc, r, vx, vy, vz, em);
+    }
+    if (J2 && j2) {
+      const T* stp = P.state + (long long)(r * P.nst) * nvox + v;
+      T st[7], de[6], d6[6];
+#pragma unroll
+      for (int c = 0; c < 7; ++c) st[c] = stp[c * nvox];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) de[c] = c < 3 ? em[c] : T(0.5) * em[c];
+      j2_strain<T>(lc, de, st, d6, p6, nullptr);
+    } else {
+      elastic_strain<T, 1>(law, lc, lm, one(em), one(p6));
+    }
+    *spv += norm6<T>(p6);
+    T* base = P.vs + (size_t)(r * 6) * nvox + v;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = p6[c];
+  }
+}
+
+// Blocks a SM keeps of the two-pass residual's kernels.  FP32 with small-strain laws waits for
+// its gathers, and its general paths (quadratic mean fields, face nodes) would otherwise set the
+// registers of the plain ones: held to four blocks (64 registers) the 128^3 J2 residual measured
+// k_stress 149 -> 112 us, k_stress_inc 144 -> 129, k_div 68 -> 52 / 81 -> 65; three blocks gave
+// 120 / 141 / 56 / 73, five (spills) 159 / 141 / 51 / 64.  FP64 is bound by its pipe and the
+// finite-strain laws by their own registers: no line for them.
+template <typename T, int SL>
+constexpr int resident_blocks() { return sizeof(T) == 4 && SL < 2 ? 4 : 0; }
+
 template <typename T, int TETRA, bool WITH_P, bool LO, bool SYM, int SL>
-__global__ void __launch_bounds__(RTX * RTY) k_stress(ResParams<T> P, TileIdx ti) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(ResParams<T> P, TileIdx ti) {
   if (P.stop && *P.stop) return;
   constexpr bool J2 = (SL & 1) != 0;
   constexpr int NPP = TETRA ? 2 : 1;
@@ -845,7 +1088,7 @@ __global__ void __launch_bounds__(RTX * RTY) k_stress(ResParams<T> P, TileIdx ti
       }
       const int v = vx + vy_ * vy + vz * vz_;
       const int ph = P.phase[v];
-      const int law = __ldg(P.law_id + ph);
+      const int law = P.one_law >= 0 ? P.one_law : __ldg(P.law_id + ph);
       const bool j2 = J2 && law == LAW_J2;
       const T* lc = P.law_c + (size_t)ph * LAWC;
       if (j2) {  // J2 takes the increment since the commit (u^f_n in the problem's own layout)
@@ -861,48 +1104,52 @@ __global__ void __launch_bounds__(RTX * RTY) k_stress(ResParams<T> P, TileIdx ti
         }
       }
       T spv = T(0);
+      if (SYM && !WITH_P && P.us[0] == nullptr) {  // small-strain laws on the strain alone
+        stress_sym<T, TETRA, LO, J2>(P, law, lc, P.law_m + (size_t)ph * 36, j2, uh, ul, vx, vy_, vz, v, nvox, &spv);
+      } else {
 #pragma unroll
-      for (int r = 0; r < NPP; ++r) {
-        T Gf[9], Gt[9], Pp[9];
-        law_grad<T, TETRA, LO>(P, j2, uh, ul, r, vx, vy_, vz, Gf, Gt);
-        if (SL) point_law<T, SL>(P, law, lc, Gt, r, v, nvox, Pp, nullptr);
-        else law_eval<T>(law, lc, Gt, Pp);
-        T* base = P.vs + (size_t)(r * NCT) * nvox + v;
-        if (SYM) {
-          const T s6[6] = {Pp[0], Pp[4], Pp[8], Pp[5], Pp[2], Pp[1]};
+        for (int r = 0; r < NPP; ++r) {
+          T Gf[9], Gt[9], Pp[9];
+          law_grad<T, TETRA, LO>(P, j2, uh, ul, r, vx, vy_, vz, Gf, Gt);
+          if (SL) point_law<T, SL>(P, law, lc, Gt, r, v, nvox, Pp, nullptr);
+          else law_eval<T>(law, lc, Gt, Pp);
+          T* base = P.vs + (size_t)(r * NCT) * nvox + v;
+          if (SYM) {
+            const T s6[6] = {Pp[0], Pp[4], Pp[8], Pp[5], Pp[2], Pp[1]};
 #pragma unroll
-          for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = s6[c];
-        } else {
+            for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = s6[c];
+          } else {
 #pragma unroll
-          for (int c = 0; c < 9; ++c) base[(size_t)c * nvox] = Pp[c];
-        }
-#pragma unroll
-        for (int c = 0; c < 9; ++c) spv += Pp[c] * Pp[c];
-        if (WITH_P) {
-          if (j2) {  // tau takes grad u^f: add grad u^f_n back to the increment's gradient
-            T nh[3][8], nl[3][8], Gn[9];
-            for (int o = 0; o < 8; ++o) {
-              int gx = vx + (o & 1), gy = vy_ + ((o >> 1) & 1), gz = vz + (o >> 2);
-              if (P.periodic[0] && gx == n1) gx = 0;
-              if (P.periodic[1] && gy == n2) gy = 0;
-              if (P.periodic[2] && gz == n3) gz = 0;
-              const int at = gx + gy * sy + gz * sz;
-              for (int c = 0; c < 3; ++c) {
-                nh[c][o] = P.un[c][at];
-                nl[c][o] = LO ? P.unlo[c][at] : T(0);
-              }
-            }
-            point_grad<T, TETRA, LO>(nh, nl, r, P.wgrad, Gn);
-            for (int i = 0; i < 9; ++i) Gf[i] += Gn[i];
+            for (int c = 0; c < 9; ++c) base[(size_t)c * nvox] = Pp[c];
           }
 #pragma unroll
-          for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              T tq = P.two_mu0 * Gf[i * 3 + q] - Pp[i * 3 + q];
-              if (i == q) tq += P.lam0 * (P.c0 ? Gf[0] + Gf[4] + Gf[8] : Gf[i * 3 + i]);
-              base[(size_t)(NC + i * 3 + q) * nvox] = tq;
+          for (int c = 0; c < 9; ++c) spv += Pp[c] * Pp[c];
+          if (WITH_P) {
+            if (j2) {  // tau takes grad u^f: add grad u^f_n back to the increment's gradient
+              T nh[3][8], nl[3][8], Gn[9];
+              for (int o = 0; o < 8; ++o) {
+                int gx = vx + (o & 1), gy = vy_ + ((o >> 1) & 1), gz = vz + (o >> 2);
+                if (P.periodic[0] && gx == n1) gx = 0;
+                if (P.periodic[1] && gy == n2) gy = 0;
+                if (P.periodic[2] && gz == n3) gz = 0;
+                const int at = gx + gy * sy + gz * sz;
+                for (int c = 0; c < 3; ++c) {
+                  nh[c][o] = P.un[c][at];
+                  nl[c][o] = LO ? P.unlo[c][at] : T(0);
+                }
+              }
+              point_grad<T, TETRA, LO>(nh, nl, r, P.wgrad, Gn);
+              for (int i = 0; i < 9; ++i) Gf[i] += Gn[i];
             }
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                T tq = P.two_mu0 * Gf[i * 3 + q] - Pp[i * 3 + q];
+                if (i == q) tq += P.lam0 * (P.c0 ? Gf[0] + Gf[4] + Gf[8] : Gf[i * 3 + i]);
+                base[(size_t)(NC + i * 3 + q) * nvox] = tq;
+              }
+          }
         }
       }
       sp += spv;
@@ -922,7 +1169,7 @@ __global__ void __launch_bounds__(RTX * RTY) k_stress(ResParams<T> P, TileIdx ti
 // P - P_n, with P_n the stress at the commit (elastic laws: the law applied to the
 // gradient increment; J2: j2_inc).  S_P still takes the full P.
 template <typename T, int TETRA, bool LO, bool SYM>
-__global__ void __launch_bounds__(RTX * RTY) k_stress_inc(ResParams<T> P, TileIdx ti) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0>()) k_stress_inc(ResParams<T> P, TileIdx ti) {
   if (P.stop && *P.stop) return;
   constexpr int NPP = TETRA ? 2 : 1;
   constexpr int NC = SYM ? 6 : 9;
@@ -940,9 +1187,10 @@ __global__ void __launch_bounds__(RTX * RTY) k_stress_inc(ResParams<T> P, TileId
     if (vx < n1 && vy_ < n2) {
       const int v = vx + vy_ * vy + vz * vz_;
       const int ph = P.phase[v];
-      const int law = __ldg(P.law_id + ph);
+      const int law = P.one_law >= 0 ? P.one_law : __ldg(P.law_id + ph);
       const bool j2 = law == LAW_J2;
       const T* lc = P.law_c + (size_t)ph * LAWC;
+      const T* lm = P.law_m + (size_t)ph * 36;
       T uh[3][8], ul[3][8];
       int at[8];
 #pragma unroll
@@ -959,46 +1207,89 @@ __global__ void __launch_bounds__(RTX * RTY) k_stress_inc(ResParams<T> P, TileId
         }
       }
       T spv = T(0);
-      if (!j2) {  // |P|^2 of the elastic law on the total gradient
+      const bool strain = SYM && P.us[0] == nullptr;  // small-strain laws on the strain alone
+      if (SYM && strain) {
+        if (!j2) {
+#pragma unroll
+          for (int r = 0; r < NPP; ++r) {
+            T s[3][3], em[6], p6[6];
+            point_sums<T, TETRA, LO>(uh, ul, r, s);
+            sum_strain<T>(s, P.wgrad, P.e0, em);
+            if (P.quad) add_quad_strain<T, TETRA>(P.hh, P.Qc, r, vx, vy_, vz, em);
+            elastic_strain<T, 1>(law, lc, lm, one(em), one(p6));
+            spv += norm6<T>(p6);
+          }
+        }
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            uh[c][o] -= __ldg(P.un[c] + at[o]);
+            if (LO) ul[c][o] -= __ldg(P.unlo[c] + at[o]);
+          }
 #pragma unroll
         for (int r = 0; r < NPP; ++r) {
-          T Gf[9], Gt[9], Pp[9];
-          law_grad<T, TETRA, LO>(P, false, uh, ul, r, vx, vy_, vz, Gf, Gt);
-          law_eval<T>(law, lc, Gt, Pp);
+          T s[3][3], em[6], d6[6];
+          point_sums<T, TETRA, LO>(uh, ul, r, s);
+          sum_strain<T>(s, P.wgrad, P.de0, em);
+          if (P.dquad) add_quad_strain<T, TETRA>(P.hh, P.dQ, r, vx, vy_, vz, em);
+          if (j2) {
+            const T* stp = P.state + (long long)(r * P.nst) * nvox + v;
+            T st[7], de[6], p6[6];
 #pragma unroll
-          for (int c = 0; c < 9; ++c) spv += Pp[c] * Pp[c];
+            for (int c = 0; c < 7; ++c) st[c] = stp[c * nvox];
+            for (int c = 0; c < 6; ++c) de[c] = c < 3 ? em[c] : T(0.5) * em[c];
+            j2_strain<T>(lc, de, st, d6, p6, nullptr);
+            spv += norm6<T>(p6);
+          } else {
+            elastic_strain<T, 1>(law, lc, lm, one(em), one(d6));
+          }
+          T* base = P.vs + (size_t)(r * 6) * nvox + v;
+#pragma unroll
+          for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = d6[c];
         }
-      }
+      } else {
+        if (!j2) {  // |P|^2 of the elastic law on the total gradient
 #pragma unroll
-      for (int o = 0; o < 8; ++o)
+          for (int r = 0; r < NPP; ++r) {
+            T Gf[9], Gt[9], Pp[9];
+            law_grad<T, TETRA, LO>(P, false, uh, ul, r, vx, vy_, vz, Gf, Gt);
+            law_eval<T>(law, lc, Gt, Pp);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          uh[c][o] -= __ldg(P.un[c] + at[o]);
-          if (LO) ul[c][o] -= __ldg(P.unlo[c] + at[o]);
+            for (int c = 0; c < 9; ++c) spv += Pp[c] * Pp[c];
+          }
         }
 #pragma unroll
-      for (int r = 0; r < NPP; ++r) {
-        T Gd[9], dG[9], dP[9];
-        law_grad<T, TETRA, LO>(P, true, uh, ul, r, vx, vy_, vz, Gd, dG);
-        if (j2) {
-          const T* stp = P.state + (long long)(r * P.nst) * nvox + v;
-          T st[7], Pf[9];
+        for (int o = 0; o < 8; ++o)
 #pragma unroll
-          for (int c = 0; c < 7; ++c) st[c] = stp[c * nvox];
-          j2_inc<T>(lc, dG, st, dP, Pf, nullptr);
+          for (int c = 0; c < 3; ++c) {
+            uh[c][o] -= __ldg(P.un[c] + at[o]);
+            if (LO) ul[c][o] -= __ldg(P.unlo[c] + at[o]);
+          }
 #pragma unroll
-          for (int c = 0; c < 9; ++c) spv += Pf[c] * Pf[c];
-        } else {
-          law_eval<T>(law, lc, dG, dP);
-        }
-        T* base = P.vs + (size_t)(r * NC) * nvox + v;
-        if (SYM) {
-          const T s6[6] = {dP[0], dP[4], dP[8], dP[5], dP[2], dP[1]};
+        for (int r = 0; r < NPP; ++r) {
+          T Gd[9], dG[9], dP[9];
+          law_grad<T, TETRA, LO>(P, true, uh, ul, r, vx, vy_, vz, Gd, dG);
+          if (j2) {
+            const T* stp = P.state + (long long)(r * P.nst) * nvox + v;
+            T st[7], Pf[9];
 #pragma unroll
-          for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = s6[c];
-        } else {
+            for (int c = 0; c < 7; ++c) st[c] = stp[c * nvox];
+            j2_inc<T>(lc, dG, st, dP, Pf, nullptr);
 #pragma unroll
-          for (int c = 0; c < 9; ++c) base[(size_t)c * nvox] = dP[c];
+            for (int c = 0; c < 9; ++c) spv += Pf[c] * Pf[c];
+          } else {
+            law_eval<T>(law, lc, dG, dP);
+          }
+          T* base = P.vs + (size_t)(r * NC) * nvox + v;
+          if (SYM) {
+            const T s6[6] = {dP[0], dP[4], dP[8], dP[5], dP[2], dP[1]};
+#pragma unroll
+            for (int c = 0; c < 6; ++c) base[(size_t)c * nvox] = s6[c];
+          } else {
+#pragma unroll
+            for (int c = 0; c < 9; ++c) base[(size_t)c * nvox] = dP[c];
+          }
         }
       }
       sp += spv;
@@ -1131,7 +1422,7 @@ __device__ __forceinline__ T store_node(const ResParams<T>& P, int mx, int my, i
 // (43 -> 16 us at 32^3 in FP64, where a thread used to walk an interior node and then a face
 // node with its three components in turn).
 template <typename T, int TETRA, bool WITH_P, bool SYM, bool INC>
-__global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0>()) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
   if (P.stop && *P.stop) return;
   constexpr int NC = SYM ? 6 : 9;
   constexpr int NCT = WITH_P ? NC + 9 : NC;
@@ -1176,34 +1467,42 @@ __global__ void __launch_bounds__(RTX * RTY) k_div(ResParams<T> P, TileIdx ti, F
         if (vz < 0) vz += n3;
         vidx[o] = vx + vyy * vy + vz * vz_;
       }
+      if constexpr (SYM && !WITH_P) {
+        sym_div<T>([&](int c, int o) {
+          // odd-parity corner -> T1 point, even -> T2 point (HEX1: the single point)
+          const bool odd = ((o ^ (o >> 1) ^ (o >> 2)) & 1) != 0;
+          return __ldg(P.vs + (size_t)((TETRA && !odd ? NC : 0) + c) * nvox + vidx[o]);
+        }, P.wdiv, Dq);
+      } else {
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < 3; ++i) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const int c = SYM ? sym_index(i, q) : i * 3 + q;
-          const T* b0 = P.vs + (size_t)c * nvox;                  // T1 point
-          const T* b1 = P.vs + (size_t)(NCT + c) * nvox;          // T2 point
-          const T* t0 = P.vs + (size_t)(NC + i * 3 + q) * nvox;   // tau, T1
-          const T* t1 = P.vs + (size_t)(NCT + NC + i * 3 + q) * nvox;
-          T s = T(0), st = T(0);
+          for (int q = 0; q < 3; ++q) {
+            const int c = SYM ? sym_index(i, q) : i * 3 + q;
+            const T* b0 = P.vs + (size_t)c * nvox;                  // T1 point
+            const T* b1 = P.vs + (size_t)(NCT + c) * nvox;          // T2 point
+            const T* t0 = P.vs + (size_t)(NC + i * 3 + q) * nvox;   // tau, T1
+            const T* t1 = P.vs + (size_t)(NCT + NC + i * 3 + q) * nvox;
+            T s = T(0), st = T(0);
 #pragma unroll
-          for (int o = 0; o < 8; ++o) {
-            if ((o >> i) & 1) continue;
-            const int o1 = o | (1 << i);
-            // odd-parity corner -> T1 point, even -> T2 point (HEX1: the single point)
-            const bool odd0 = (((o & 1) + ((o >> 1) & 1) + (o >> 2)) & 1) != 0;
-            const bool odd1 = !odd0;
-            const T* p0 = (!TETRA || odd0) ? b0 : b1;
-            const T* p1 = (!TETRA || odd1) ? b0 : b1;
-            s += __ldg(p1 + vidx[o1]) - __ldg(p0 + vidx[o]);
-            if (WITH_P) {
-              const T* q0 = (!TETRA || odd0) ? t0 : t1;
-              const T* q1 = (!TETRA || odd1) ? t0 : t1;
-              st += __ldg(q1 + vidx[o1]) - __ldg(q0 + vidx[o]);
+            for (int o = 0; o < 8; ++o) {
+              if ((o >> i) & 1) continue;
+              const int o1 = o | (1 << i);
+              // odd-parity corner -> T1 point, even -> T2 point (HEX1: the single point)
+              const bool odd0 = (((o & 1) + ((o >> 1) & 1) + (o >> 2)) & 1) != 0;
+              const bool odd1 = !odd0;
+              const T* p0 = (!TETRA || odd0) ? b0 : b1;
+              const T* p1 = (!TETRA || odd1) ? b0 : b1;
+              s += __ldg(p1 + vidx[o1]) - __ldg(p0 + vidx[o]);
+              if (WITH_P) {
+                const T* q0 = (!TETRA || odd0) ? t0 : t1;
+                const T* q1 = (!TETRA || odd1) ? t0 : t1;
+                st += __ldg(q1 + vidx[o1]) - __ldg(q0 + vidx[o]);
+              }
             }
+            Dq[q] += P.wdiv[i] * s;
+            if (WITH_P) pq[q] += P.wdiv[i] * st;
           }
-          Dq[q] += P.wdiv[i] * s;
-          if (WITH_P) pq[q] += P.wdiv[i] * st;
         }
       }
       sd += store_node<T, WITH_P, INC>(P, mx, my, mz, Dq, pq);
@@ -1322,129 +1621,6 @@ static FusedGeom fused_geom(const ResParams<T>& P) {
   return g;
 }
 
-// The first 24 coefficients of a phase's law row (isotropic: lambda, mu; cubic: the upper
-// triangle of the rotated Mandel stiffness, 21 entries), loaded together as vectors.
-template <typename T>
-__device__ __forceinline__ void load_law24(const T* __restrict__ lc, T c[24]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4* v = reinterpret_cast<const float4*>(lc);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const float4 a = __ldg(v + i);
-      c[4 * i] = a.x; c[4 * i + 1] = a.y; c[4 * i + 2] = a.z; c[4 * i + 3] = a.w;
-    }
-  } else {
-    const double2* v = reinterpret_cast<const double2*>(lc);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) {
-      const double2 a = __ldg(v + i);
-      c[2 * i] = a.x; c[2 * i + 1] = a.y;
-    }
-  }
-}
-
-// Small-strain elastic law from coefficients in registers: P as (11, 22, 33, 23, 13, 12).
-template <typename T>
-__device__ __forceinline__ void elastic_reg(int law, const T c[24], const T G[9], T s[6]) {
-  const T e00 = G[0], e11 = G[4], e22 = G[8];
-  const T e12 = T(0.5) * (G[5] + G[7]), e02 = T(0.5) * (G[2] + G[6]), e01 = T(0.5) * (G[1] + G[3]);
-  if (law == LAW_CUBIC) {
-    const T r2 = T(1.41421356237309504880), ir2 = T(0.70710678118654752440);
-    const T em[6] = {e00, e11, e22, r2 * e12, r2 * e02, r2 * e01};
-    T sm[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    int k = 0;
-#pragma unroll
-    for (int a = 0; a < 6; ++a)
-#pragma unroll
-      for (int b = a; b < 6; ++b) {
-        const T v = c[k++];
-        sm[a] += v * em[b];
-        if (b != a) sm[b] += v * em[a];
-      }
-    s[0] = sm[0]; s[1] = sm[1]; s[2] = sm[2];
-    s[3] = ir2 * sm[3]; s[4] = ir2 * sm[4]; s[5] = ir2 * sm[5];
-  } else {  // isotropic
-    const T mu2 = T(2) * c[1], tr = c[0] * (e00 + e11 + e22);
-    s[0] = tr + mu2 * e00; s[1] = tr + mu2 * e11; s[2] = tr + mu2 * e22;
-    s[3] = mu2 * e12; s[4] = mu2 * e02; s[5] = mu2 * e01;
-  }
-}
-
-// Gradient at point r from the corner values of the lower (L, corners o < 4) and upper
-// (U, corners o >= 4) node planes, as point_grad forms it.  The FP32 variant takes (hi, lo)
-// pairs and uses packed FP32x2 arithmetic (one instruction per pair) with the same
-// differences, sums and rounding.
-template <int TETRA>
-__device__ __forceinline__ void grad_lu_f2(const float2 L[3][4], const float2 U[3][4], int r, const float* wg,
-                                           float G[9]) {
-  const float2 m1 = make_float2(-1.f, -1.f);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const int mask = TETRA ? ((1 << i) | (1 << ((i + 1) % 3))) : (1 << i);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      float2 s = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        if ((o >> i) & 1) continue;
-        const int par = ((o & 1) + ((o >> 1) & 1) + ((o >> 2) & 1)) & 1;
-        if (TETRA && ((r == 0) != (par == 0))) continue;
-        const int o2 = o ^ mask;
-        const float2 a = o < 4 ? L[q][o] : U[q][o - 4];
-        const float2 b = o2 < 4 ? L[q][o2] : U[q][o2 - 4];
-        s = __fadd2_rn(s, __ffma2_rn(a, m1, b));  // + (u(o ^ mask) - u(o))
-      }
-      G[i * 3 + q] = wg[i] * (s.x + s.y);
-    }
-  }
-}
-
-template <typename T, int TETRA>
-__device__ __forceinline__ void grad_lu(const T L[3][4], const T U[3][4], int r, const T* wg, T G[9]) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const int mask = TETRA ? ((1 << i) | (1 << ((i + 1) % 3))) : (1 << i);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      T s = T(0);
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        if ((o >> i) & 1) continue;
-        const int par = ((o & 1) + ((o >> 1) & 1) + ((o >> 2) & 1)) & 1;
-        if (TETRA && ((r == 0) != (par == 0))) continue;
-        const int o2 = o ^ mask;
-        s += (o2 < 4 ? L[q][o2] : U[q][o2 - 4]) - (o < 4 ? L[q][o] : U[q][o - 4]);
-      }
-      G[i * 3 + q] = wg[i] * s;
-    }
-  }
-}
-
-// Small-strain elastic law with the phase's full Mandel stiffness (9 blocks of 2 x 2, see
-// ResParams::law_m) and packed FP32x2 products: P as (11, 22, 33, 23, 13, 12).
-__device__ __forceinline__ void elastic_f2(const float4* __restrict__ M4, const float G[9], float s[6]) {
-  const float r2 = 1.41421356237309504880f, ir2 = 0.70710678118654752440f;
-  const float em[6] = {G[0], G[4], G[8], r2 * (0.5f * (G[5] + G[7])), r2 * (0.5f * (G[2] + G[6])),
-                       r2 * (0.5f * (G[1] + G[3]))};
-  float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-  for (int bp = 0; bp < 3; ++bp) {
-    const float2 e0 = make_float2(em[2 * bp], em[2 * bp]), e1 = make_float2(em[2 * bp + 1], em[2 * bp + 1]);
-#pragma unroll
-    for (int rp = 0; rp < 3; ++rp) {
-      const float4 c = __ldg(M4 + 3 * bp + rp);
-      acc[rp] = __ffma2_rn(make_float2(c.x, c.y), e0, acc[rp]);
-      acc[rp] = __ffma2_rn(make_float2(c.z, c.w), e1, acc[rp]);
-    }
-  }
-  s[0] = acc[0].x;
-  s[1] = acc[0].y;
-  s[2] = acc[1].x;
-  s[3] = ir2 * acc[1].y;
-  s[4] = ir2 * acc[2].x;
-  s[5] = ir2 * acc[2].y;
-}
-
 template <int V> struct Par { static constexpr int value = V; };
 
 template <typename T, int TETRA, bool LO, int FY>
@@ -1554,43 +1730,38 @@ __global__ void __launch_bounds__(FX * FY, 16 / FY) k_residual_fused(ResParams<T
   auto voxel_layer = [&](int b, int vz, int ph, const NV (&L)[3][4], const NV (&U)[3][4]) {
     const bool zin = vz >= 0 && vz < n3;
     const int vzz = vz < 0 ? vz + n3 : vz;
-    T Ps[NPP][6];
+    T Ps[NPP][6], spv = T(0);
 #pragma unroll
     for (int r = 0; r < NPP; ++r)
 #pragma unroll
       for (int c = 0; c < 6; ++c) Ps[r][c] = T(0);
     if (vin && (zin || P.periodic[2])) {
-      if constexpr (LO) {  // FP32 hi + lo fields: packed FP32x2 gradient and law
-        const float4* M4 = reinterpret_cast<const float4*>(P.law_m + (size_t)ph * 36);
+      const T* lm = P.law_m + (size_t)ph * 36;
+      const int law = P.one_law >= 0 ? P.one_law : __ldg(P.law_id + ph);
+      const T* lc = P.law_c + (size_t)ph * LAWC;
+      T em[NPP][6];
 #pragma unroll
-        for (int r = 0; r < NPP; ++r) {
-          float Gf[9], Gt[9];
-          grad_lu_f2<TETRA>(L, U, r, P.wgrad, Gf);
+      for (int r = 0; r < NPP; ++r) {
+        T sums[3][3];
 #pragma unroll
-          for (int i = 0; i < 9; ++i) Gt[i] = Gf[i] + P.Gs[i];
-          if (P.quad) add_quad<T, TETRA>(P.hh, P.Qc, r, vx, vy, vzz, Gt);
-          elastic_f2(M4, Gt, Ps[r]);
+        for (int q = 0; q < 3; ++q) {
+          auto u = [&](int o) { return o < 4 ? L[q][o] : U[q][o - 4]; };
+          if constexpr (LO) {
+            float2 t[3];
+            corner_diffs<PairOps, TETRA, float2>(u, r, t);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) sums[q][i] = t[i].x + t[i].y;
+          } else {
+            corner_diffs<ScalarOps, TETRA, T>(u, r, sums[q]);
+          }
         }
-      } else {
-        const int law = __ldg(P.law_id + ph);
-        T lc[24];
-        load_law24<T>(P.law_c + (size_t)ph * LAWC, lc);
-#pragma unroll
-        for (int r = 0; r < NPP; ++r) {
-          T Gf[9], Gt[9];
-          grad_lu<T, TETRA>(L, U, r, P.wgrad, Gf);
-#pragma unroll
-          for (int i = 0; i < 9; ++i) Gt[i] = Gf[i] + P.Gs[i];
-          if (P.quad) add_quad<T, TETRA>(P.hh, P.Qc, r, vx, vy, vzz, Gt);
-          elastic_reg<T>(law, lc, Gt, Ps[r]);
-        }
+        sum_strain<T>(sums, P.wgrad, P.e0, em[r]);
+        if (P.quad) add_quad_strain<T, TETRA>(P.hh, P.Qc, r, vx, vy, vzz, em[r]);
       }
-      if (own_xy && vz >= own_z0 && vz < Z1) {
-        T spv = T(0);
+      elastic_strain<T, NPP>(law, lc, lm, em, Ps);
 #pragma unroll
-        for (int r = 0; r < NPP; ++r)
-          spv += Ps[r][0] * Ps[r][0] + Ps[r][1] * Ps[r][1] + Ps[r][2] * Ps[r][2] +
-                 T(2) * (Ps[r][3] * Ps[r][3] + Ps[r][4] * Ps[r][4] + Ps[r][5] * Ps[r][5]);
+      for (int r = 0; r < NPP; ++r) spv += norm6<T>(Ps[r]);
+      if (own_xy && vz >= own_z0 && vz < Z1) {
         sp += spv;
         if (g.faces && (xy_face || (g.fdof[2] && (vzz == 0 || vzz == n3 - 1)))) {
           const long long v = phase_xy + (long long)vzz * P.vz;
@@ -1628,20 +1799,8 @@ __global__ void __launch_bounds__(FX * FY, 16 / FY) k_residual_fused(ResParams<T
       val[o][0] = a0.x; val[o][1] = a0.y; val[o][2] = a1.x;
       val[o][3] = a1.y; val[o][4] = a2.x; val[o][5] = a2.y;
     }
-    T Dq[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int c = sym_index(i, q);
-        T s = T(0);
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          if ((o >> i) & 1) continue;
-          s += val[o | (1 << i)][c] - val[o][c];
-        }
-        Dq[q] += P.wdiv[i] * s;
-      }
+    T Dq[3];
+    sym_div<T>([&](int c, int o) { return val[o][c]; }, P.wdiv, Dq);
     const long long off = node_xy + z * sz;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -1901,7 +2060,7 @@ __device__ __forceinline__ int voxel_eval(const ResParams<T>& P, int vx, int vy,
   const long long nvox = (long long)n1 * n2 * n3;
   const long long v = vx + vy * P.vy + (long long)vz * P.vz;
   const int ph = P.phase[v];
-  const int law = __ldg(P.law_id + ph);
+  const int law = P.one_law >= 0 ? P.one_law : __ldg(P.law_id + ph);
   const bool j2 = (SL & 1) && law == LAW_J2;
   const T* lc = P.law_c + (size_t)ph * LAWC;
   T uh[3][8], ul[3][8];
