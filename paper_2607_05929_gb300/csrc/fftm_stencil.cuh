@@ -183,6 +183,17 @@ __device__ __forceinline__ void compose_minus_identity(const T X[9], const T Y[9
       W[i * 3 + j] = X[i * 3 + j] + Y[i * 3 + j] + X[i * 3] * Y[j] + X[i * 3 + 1] * Y[3 + j] + X[i * 3 + 2] * Y[6 + j];
 }
 
+// Slip direction and plane normal of system s in the sample frame (R: crystal -> sample), not
+// normalised.
+template <typename T>
+__device__ __forceinline__ void fcc_system(const T Rm[9], int s, T mv[3], T nv[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    nv[i] = Rm[i * 3] * T(c_fcc_sys[s][0]) + Rm[i * 3 + 1] * T(c_fcc_sys[s][1]) + Rm[i * 3 + 2] * T(c_fcc_sys[s][2]);
+    mv[i] = Rm[i * 3] * T(c_fcc_sys[s][3]) + Rm[i * 3 + 1] * T(c_fcc_sys[s][4]) + Rm[i * 3 + 2] * T(c_fcc_sys[s][5]);
+  }
+}
+
 // One implicit increment at a voxel point (Kalidindi, Bronkhorst and Anand 1992):
 // unknown second Piola-Kirchhoff Pi (6 components 11, 22, 33, 23, 13, 12),
 //   R(Pi) = Pi - Pi_tr + sum_s dgamma_s(tau_s) C : sym(A P_s),  tau_s = Pi : P_s,
@@ -191,93 +202,95 @@ __device__ __forceinline__ void compose_minus_identity(const T X[9], const T Y[9
 // system, with backtracking on max |R|; then F^p = (1 + sum dgamma_s P_s) F^p_n,
 // Gamma += sum |dgamma_s|, P = F^e Pi F^p^-T.  State st = (F^p - 1 row-major, Gamma).
 // c = Mandel C (21), gdot0, n, tau0, tau_inf, h0, dt, R (crystal -> sample, row-major).
+//
+// Bound by latency: a chain of residuals (12 powers each), Jacobians and 6 x 6 solves.  What a
+// system needs (the symmetric Schmid tensor and C : sym(A P_s)) lies in one local array that the
+// rolled loops over the systems walk; the Jacobian and its elimination (row exchanges as selects)
+// stay in registers, and the slopes of the slip rates come from the residual's own powers.  With the
+// matrix in local memory, a second set of powers per iteration and both points of a voxel in one
+// thread, the stress kernel of a 32^3 TETRA2 FP32 polycrystal took 624 us; this takes 389.
 template <typename T>
 __device__ void cp_eval(const T* __restrict__ c, const T G[9], const T st[10], T S[9], T* stn) {
   const T gdot0 = __ldg(c + 21), nexp = __ldg(c + 22), tau0 = __ldg(c + 23), tinf = __ldg(c + 24);
   const T h0 = __ldg(c + 25), dt = __ldg(c + 26);
-  T Rm[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) Rm[i] = __ldg(c + 27 + i);
-  // Schmid tensors, symmetric parts (6 components) and full (9)
-  T sP[12][6], Pf[12][9];
   const T inv6 = T(0.40824829046386301637);  // 1 / sqrt(6)
-#pragma unroll
-  for (int s = 0; s < 12; ++s) {
-    T nv[3], mv[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      nv[i] = Rm[i * 3] * T(c_fcc_sys[s][0]) + Rm[i * 3 + 1] * T(c_fcc_sys[s][1]) + Rm[i * 3 + 2] * T(c_fcc_sys[s][2]);
-      mv[i] = Rm[i * 3] * T(c_fcc_sys[s][3]) + Rm[i * 3 + 1] * T(c_fcc_sys[s][4]) + Rm[i * 3 + 2] * T(c_fcc_sys[s][5]);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Pf[s][i * 3 + j] = inv6 * mv[i] * nv[j];
-    sP[s][0] = Pf[s][0];
-    sP[s][1] = Pf[s][4];
-    sP[s][2] = Pf[s][8];
-    sP[s][3] = T(0.5) * (Pf[s][5] + Pf[s][7]);
-    sP[s][4] = T(0.5) * (Pf[s][2] + Pf[s][6]);
-    sP[s][5] = T(0.5) * (Pf[s][1] + Pf[s][3]);
-  }
   // trial elastic state: W = F F^p_n^-1 - 1, E_tr = (W + W^T + W^T W) / 2, A = 1 + 2 E_tr
-  T H[9], Y[9], W[9];
+  T H[9];
 #pragma unroll
   for (int q = 0; q < 3; ++q)
 #pragma unroll
     for (int i = 0; i < 3; ++i) H[q * 3 + i] = G[i * 3 + q];
-  inv_minus_identity<T>(st, Y);
-  compose_minus_identity<T>(H, Y, W);
-  auto ew = [&](int i, int j) {
-    return T(0.5) * (W[i * 3 + j] + W[j * 3 + i] + W[i] * W[j] + W[3 + i] * W[3 + j] + W[6 + i] * W[6 + j]);
-  };
-  const T Etr[6] = {ew(0, 0), ew(1, 1), ew(2, 2), ew(1, 2), ew(0, 2), ew(0, 1)};
   T Ptr[6];
-  mandel_apply<T>(c, Etr, Ptr);
-  // C : sym(A P_s) = C : sym(P_s) + 2 C : sym(E_tr P_s)
-  T Cs[12][6];
+  T Q[12][12];  // per system: sym(P_s) (6 components), C : sym(A P_s)
   {
-    const T Em[3][3] = {{Etr[0], Etr[5], Etr[4]}, {Etr[5], Etr[1], Etr[3]}, {Etr[4], Etr[3], Etr[2]}};
+    T Rm[9];
 #pragma unroll
+    for (int i = 0; i < 9; ++i) Rm[i] = __ldg(c + 27 + i);
+    T Y[9], W[9];
+    inv_minus_identity<T>(st, Y);
+    compose_minus_identity<T>(H, Y, W);
+    auto ew = [&](int i, int j) {
+      return T(0.5) * (W[i * 3 + j] + W[j * 3 + i] + W[i] * W[j] + W[3 + i] * W[3 + j] + W[6 + i] * W[6 + j]);
+    };
+    const T Etr[6] = {ew(0, 0), ew(1, 1), ew(2, 2), ew(1, 2), ew(0, 2), ew(0, 1)};
+    mandel_apply<T>(c, Etr, Ptr);
+    // C : sym(A P_s) = C : sym(P_s) + 2 C : sym(E_tr P_s)
+    const T Em[3][3] = {{Etr[0], Etr[5], Etr[4]}, {Etr[5], Etr[1], Etr[3]}, {Etr[4], Etr[3], Etr[2]}};
+#pragma unroll 1
     for (int s = 0; s < 12; ++s) {
-      T B[3][3];
+      T mv[3], nv[3], Pf[9], B[3][3], cs[6];
+      fcc_system<T>(Rm, s, mv, nv);
 #pragma unroll
       for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-          B[i][j] = Em[i][0] * Pf[s][j] + Em[i][1] * Pf[s][3 + j] + Em[i][2] * Pf[s][6 + j];
-      const T v[6] = {sP[s][0] + T(2) * B[0][0], sP[s][1] + T(2) * B[1][1], sP[s][2] + T(2) * B[2][2],
-                      sP[s][3] + (B[1][2] + B[2][1]), sP[s][4] + (B[0][2] + B[2][0]), sP[s][5] + (B[0][1] + B[1][0])};
-      mandel_apply<T>(c, v, Cs[s]);
+        for (int j = 0; j < 3; ++j) Pf[i * 3 + j] = inv6 * mv[i] * nv[j];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) B[i][j] = Em[i][0] * Pf[j] + Em[i][1] * Pf[3 + j] + Em[i][2] * Pf[6 + j];
+      const T sp[6] = {Pf[0], Pf[4], Pf[8], T(0.5) * (Pf[5] + Pf[7]), T(0.5) * (Pf[2] + Pf[6]), T(0.5) * (Pf[1] + Pf[3])};
+      const T v[6] = {sp[0] + T(2) * B[0][0], sp[1] + T(2) * B[1][1], sp[2] + T(2) * B[2][2],
+                      sp[3] + (B[1][2] + B[2][1]), sp[4] + (B[0][2] + B[2][0]), sp[5] + (B[0][1] + B[1][0])};
+      mandel_apply<T>(c, v, cs);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        Q[s][k] = sp[k];
+        Q[s][6 + k] = cs[k];
+      }
     }
   }
   const T gam_n = st[9];
   const T tauc = tinf > tau0 ? tau0 + (tinf - tau0) * (T(1) - exp(-h0 * gam_n / (tinf - tau0))) : tau0;
-  auto tau_of = [&](const T Pi[6], int s) {
-    return Pi[0] * sP[s][0] + Pi[1] * sP[s][1] + Pi[2] * sP[s][2] +
-           T(2) * (Pi[3] * sP[s][3] + Pi[4] * sP[s][4] + Pi[5] * sP[s][5]);
+  const T dtg = dt * gdot0;
+  auto tau_of = [&](const T Pi[6], const T* q) {
+    return Pi[0] * q[0] + Pi[1] * q[1] + Pi[2] * q[2] + T(2) * (Pi[3] * q[3] + Pi[4] * q[4] + Pi[5] * q[5]);
   };
-  auto slip = [&](T tau, T* ddg) {
+  // the slip increment at resolved shear tau, and |tau / tau_c|^(n-1)
+  auto slip = [&](T tau, T* pw) {
     const T x = tau / tauc, ax = fabs(x);
-    const T pw = ax > T(0) ? exp((nexp - T(1)) * log(ax)) : T(0);  // |x|^(n-1)
-    if (ddg) *ddg = dt * gdot0 * nexp * pw / tauc;
-    return copysign(dt * gdot0 * pw * ax, x);
+    *pw = ax > T(0) ? exp((nexp - T(1)) * log(ax)) : T(0);
+    return copysign(dtg * *pw * ax, x);
   };
+  T pw[12];  // of the systems at the last residual's stress
   auto resid = [&](const T Pi[6], T R[6]) {
     T m = T(0);
 #pragma unroll
     for (int k = 0; k < 6; ++k) R[k] = Pi[k] - Ptr[k];
+#pragma unroll 3
     for (int s = 0; s < 12; ++s) {
-      const T dg = slip(tau_of(Pi, s), nullptr);
+      T p;
+      const T dg = slip(tau_of(Pi, Q[s]), &p);
+      pw[s] = p;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) R[k] += dg * Cs[s][k];
+      for (int k = 0; k < 6; ++k) R[k] += dg * Q[s][6 + k];
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) m = fmax(m, fabs(R[k]));
     return m;
   };
   T taumax = T(0), scale = tauc;
-  for (int s = 0; s < 12; ++s) taumax = fmax(taumax, fabs(tau_of(Ptr, s)));
+#pragma unroll 3
+  for (int s = 0; s < 12; ++s) taumax = fmax(taumax, fabs(tau_of(Ptr, Q[s])));
 #pragma unroll
   for (int k = 0; k < 6; ++k) scale = fmax(scale, fabs(Ptr[k]));
   const T s0 = taumax > tauc ? tauc / taumax : T(1);
@@ -288,8 +301,9 @@ __device__ void cp_eval(const T* __restrict__ c, const T G[9], const T st[10], T
   // FP32: about two units in the last place of the largest stress component, the level at
   // which the residual itself is rounding; FP64: the oracle's tolerance
   const T tol = (sizeof(T) == 8 ? T(1e-12) : T(1.2e-7)) * scale;
+#pragma unroll 1
   for (int it = 0; it < 200 && rn > tol; ++it) {
-    // Jacobian: 1 + sum_s ddgamma_s C_s (x) dtau_s/dPi
+    // Jacobian: 1 + sum_s ddgamma_s C_s (x) dtau_s/dPi, ddgamma_s = dt gdot0 n |.|^(n-1) / tau_c
     T J[6][7];
 #pragma unroll
     for (int a = 0; a < 6; ++a) {
@@ -297,41 +311,48 @@ __device__ void cp_eval(const T* __restrict__ c, const T G[9], const T st[10], T
       for (int b = 0; b < 6; ++b) J[a][b] = (a == b) ? T(1) : T(0);
       J[a][6] = -R[a];
     }
+#pragma unroll 2
     for (int s = 0; s < 12; ++s) {
-      T ddg;
-      slip(tau_of(Pi, s), &ddg);
-      const T g[6] = {sP[s][0], sP[s][1], sP[s][2], T(2) * sP[s][3], T(2) * sP[s][4], T(2) * sP[s][5]};
+      const T ddg = dtg * nexp * pw[s] / tauc;
+      const T* q = Q[s];
+      const T g[6] = {q[0], q[1], q[2], T(2) * q[3], T(2) * q[4], T(2) * q[5]};
 #pragma unroll
       for (int a = 0; a < 6; ++a)
 #pragma unroll
-        for (int b = 0; b < 6; ++b) J[a][b] += ddg * Cs[s][a] * g[b];
+        for (int b = 0; b < 6; ++b) J[a][b] += ddg * q[6 + a] * g[b];
     }
-    // Gaussian elimination with partial pivoting
+    // Gaussian elimination with partial pivoting (the largest entry brought up row by row)
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      int piv = k;
-      for (int a = k + 1; a < 6; ++a)
-        if (fabs(J[a][k]) > fabs(J[piv][k])) piv = a;
-      if (piv != k)
-        for (int b = 0; b < 7; ++b) {
-          const T t = J[k][b];
-          J[k][b] = J[piv][b];
-          J[piv][b] = t;
+#pragma unroll
+      for (int a = k + 1; a < 6; ++a) {
+        const bool up = fabs(J[a][k]) > fabs(J[k][k]);
+#pragma unroll
+        for (int b = k; b < 7; ++b) {
+          const T u = J[k][b], v = J[a][b];
+          J[k][b] = up ? v : u;
+          J[a][b] = up ? u : v;
         }
+      }
       const T ip = T(1) / J[k][k];
+#pragma unroll
       for (int a = k + 1; a < 6; ++a) {
         const T f = J[a][k] * ip;
-        for (int b = k; b < 7; ++b) J[a][b] -= f * J[k][b];
+#pragma unroll
+        for (int b = k + 1; b < 7; ++b) J[a][b] -= f * J[k][b];
       }
     }
     T d[6];
+#pragma unroll
     for (int k = 5; k >= 0; --k) {
       T v = J[k][6];
+#pragma unroll
       for (int b = k + 1; b < 6; ++b) v -= J[k][b] * d[b];
       d[k] = v / J[k][k];
     }
     // backtracking on max |R|
     T step = T(1), Pn[6], Rn[6], rnew = rn;
+#pragma unroll 1
     for (int bt = 0; bt < (sizeof(T) == 8 ? 60 : 24); ++bt) {
 #pragma unroll
       for (int k = 0; k < 6; ++k) Pn[k] = Pi[k] + step * d[k];
@@ -349,11 +370,21 @@ __device__ void cp_eval(const T* __restrict__ c, const T G[9], const T st[10], T
   }
   // plastic update: K' = (1 + L)(1 + K) - 1, L = sum dgamma_s P_s; Gamma += sum |dgamma_s|
   T L[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)}, dgam = T(0);
-  for (int s = 0; s < 12; ++s) {
-    const T dg = slip(tau_of(Pi, s), nullptr);
-    dgam += fabs(dg);
+  {
+    T Rm[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) L[i] += dg * Pf[s][i];
+    for (int i = 0; i < 9; ++i) Rm[i] = __ldg(c + 27 + i);
+#pragma unroll 1
+    for (int s = 0; s < 12; ++s) {
+      T mv[3], nv[3], p;
+      fcc_system<T>(Rm, s, mv, nv);
+      const T dg = slip(tau_of(Pi, Q[s]), &p);
+      dgam += fabs(dg);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) L[i * 3 + j] += dg * (inv6 * mv[i] * nv[j]);
+    }
   }
   T K1[9], Y1[9], W1[9];
   compose_minus_identity<T>(L, st, K1);
@@ -380,33 +411,59 @@ __device__ void cp_eval(const T* __restrict__ c, const T G[9], const T st[10], T
 }
 
 // Eigen-decomposition of a symmetric 3x3 tensor A (11, 22, 33, 23, 13, 12) by cyclic
-// Jacobi rotations (each rotation zeroes one off-diagonal entry; the tangent of the angle is
-// taken as the smaller root of t^2 + 2 th t - 1 = 0, th = (a_qq - a_pp) / (2 a_pq), and the
-// other entries are updated through tau = s / (1 + c) to limit cancellation).  Returns the
-// eigenvalues w and the eigenvectors as the columns of V (row-major).  The sweep count is
-// fixed: convergence is quadratic, so 5 (FP32) or 6 (FP64) sweeps leave the off-diagonal at
-// rounding level for any input; an entry that is already zero is skipped.
+// Jacobi rotations: each rotation zeroes one off-diagonal entry b between diagonal entries whose
+// half difference is d, by the angle of tangent t = b sign(d) / h, h = |d| + sqrt(d^2 + b^2) (the
+// smaller root), cosine h / sqrt(h^2 + b^2); the other entries are updated through
+// tau = s / (1 + c) to limit cancellation.  Returns the eigenvalues w and the eigenvectors as the
+// columns of V (row-major).  The tensor is scaled by a power of two to order one first, so that the
+// squares neither underflow nor overflow; the sweeps end when every off-diagonal entry lies below a
+// quarter unit of the largest one (convergence is quadratic: four sweeps as a rule), an entry that is
+// already below is skipped.  Bound by the FP64 pipe: a fixed six sweeps of four divisions and two
+// square roots per rotation cost half of the law (48^3 TETRA2 stress kernel: 1117 us, now 624).
 template <typename T>
 __host__ __device__ void sym_eig3(const T A6[6], T w[3], T V[9]) {
   T a[3][3] = {{A6[0], A6[5], A6[4]}, {A6[5], A6[1], A6[3]}, {A6[4], A6[3], A6[2]}};
 #pragma unroll
   for (int i = 0; i < 9; ++i) V[i] = (i % 4 == 0) ? T(1) : T(0);
-  constexpr int SWEEPS = sizeof(T) == 8 ? 6 : 5;
+  constexpr int SWEEPS = sizeof(T) == 8 ? 6 : 5, LOWE = sizeof(T) == 8 ? -1022 : -126;
+  const T small = sizeof(T) == 8 ? T(2.7755575615628914e-17) : T(1.4901161193847656e-08);  // 2^-55, 2^-26
+  T big = T(0);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) big = fmax(big, fabs(A6[k]));
+  T back = T(1);
+  if (big > T(0) && big < (sizeof(T) == 8 ? T(1e300) : T(1e37))) {
+    const int e = ilogb(big) < LOWE ? LOWE : ilogb(big);  // 2^e and 2^-e are normal numbers
+    const T sc = scalbn(T(1), -e);
+    back = scalbn(T(1), e);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) a[i][j] *= sc;
+    big *= sc;
+  }
+  const T tiny = small * big;
   for (int sw = 0; sw < SWEEPS; ++sw) {
+    if (fabs(a[0][1]) <= tiny && fabs(a[0][2]) <= tiny && fabs(a[1][2]) <= tiny) break;  // (false for a NaN)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const int p = k == 2 ? 1 : 0, q = k == 0 ? 1 : 2, r = 3 - p - q;
-      const T apq = a[p][q];
-      if (apq == T(0)) continue;
-      const T th = (a[q][q] - a[p][p]) / (T(2) * apq);
-      const T t = copysign(T(1), th) / (fabs(th) + sqrt(th * th + T(1)));  // th^2 = inf gives t = 0
-      const T c = T(1) / sqrt(t * t + T(1)), sn = t * c, tau = sn / (T(1) + c);
-      a[p][p] -= t * apq;
-      a[q][q] += t * apq;
+      const T b = a[p][q];
+      if (fabs(b) <= tiny) continue;
+      const T d = T(0.5) * (a[q][q] - a[p][p]);
+      const T h = fabs(d) + sqrt(d * d + b * b);
+      const T t = copysign(T(1), d) * b / h;
+#ifdef __CUDA_ARCH__
+      const T inv = rsqrt(h * h + b * b);
+#else
+      const T inv = T(1) / sqrt(h * h + b * b);
+#endif
+      const T c = h * inv, sn = copysign(T(1), d) * b * inv, tau = sn / (T(1) + c);
+      a[p][p] -= t * b;
+      a[q][q] += t * b;
       a[p][q] = a[q][p] = T(0);
-      const T g = a[r][p], h = a[r][q];
-      a[r][p] = a[p][r] = g - sn * (h + g * tau);
-      a[r][q] = a[q][r] = h + sn * (g - h * tau);
+      const T g = a[r][p], u = a[r][q];
+      a[r][p] = a[p][r] = g - sn * (u + g * tau);
+      a[r][q] = a[q][r] = u + sn * (g - u * tau);
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         const T vg = V[i * 3 + p], vh = V[i * 3 + q];
@@ -415,9 +472,9 @@ __host__ __device__ void sym_eig3(const T A6[6], T w[3], T V[9]) {
       }
     }
   }
-  w[0] = a[0][0];
-  w[1] = a[1][1];
-  w[2] = a[2][2];
+  w[0] = back * a[0][0];
+  w[1] = back * a[1][1];
+  w[2] = back * a[2][2];
 }
 
 // Perfect von Mises plasticity in the logarithmic strain space (Sec. 3.2, the porous
@@ -445,12 +502,13 @@ __host__ __device__ void log_j2_eval(const T* __restrict__ c, const T G[9], cons
     hl[a] = T(0.5) * log1p(T(2) * e[a]);
   }
   constexpr int I6[6][2] = {{0, 0}, {1, 1}, {2, 2}, {1, 2}, {0, 2}, {0, 1}};
-  T He[6];
+  T He[6], Vh[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) Vh[i] = V[i] * hl[i % 3];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int i = I6[k][0], j = I6[k][1];
-    He[k] = (V[i * 3] * hl[0] * V[j * 3] + V[i * 3 + 1] * hl[1] * V[j * 3 + 1] + V[i * 3 + 2] * hl[2] * V[j * 3 + 2]) -
-            st[k];
+    He[k] = (Vh[i * 3] * V[j * 3] + Vh[i * 3 + 1] * V[j * 3 + 1] + Vh[i * 3 + 2] * V[j * 3 + 2]) - st[k];
   }
   const T tr = He[0] + He[1] + He[2], m = tr * T(1.0 / 3.0), m2 = T(2) * mu;
   const T s6[6] = {m2 * (He[0] - m), m2 * (He[1] - m), m2 * (He[2] - m), m2 * He[3], m2 * He[4], m2 * He[5]};
@@ -472,7 +530,7 @@ __host__ __device__ void log_j2_eval(const T* __restrict__ c, const T G[9], cons
   const T Tm[3][3] = {{scale * s6[0] + kt, scale * s6[5], scale * s6[4]},
                       {scale * s6[5], scale * s6[1] + kt, scale * s6[3]},
                       {scale * s6[4], scale * s6[3], scale * s6[2] + kt}};
-  // St = theta o (V^T T V), then S = V St V^T
+  // St = theta o (V^T T V), then S = V St V^T (both symmetric: six entries each)
   T TV[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -483,22 +541,26 @@ __host__ __device__ void log_j2_eval(const T* __restrict__ c, const T G[9], cons
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
+    for (int b = 0; b <= a; ++b) {
       const T tt = V[a] * TV[0][b] + V[3 + a] * TV[1][b] + V[6 + a] * TV[2][b];
-      const T r = T(2) * (e[a] - e[b]) / w[b];
-      const T th = fabs(r) < near ? T(2) / (w[a] + w[b]) : log1p(r) / (w[b] * r);
-      St[a][b] = th * tt;
+      T th;
+      if (a == b) {
+        th = T(1) / w[a];
+      } else {
+        const T r = T(2) * (e[a] - e[b]) / w[b];
+        th = fabs(r) < near ? T(2) / (w[a] + w[b]) : log1p(r) / (w[b] * r);
+      }
+      St[a][b] = St[b][a] = th * tt;
     }
-  T Pi[6];
+  T VS[3][3], Pi[6];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) VS[i][b] = V[i * 3] * St[0][b] + V[i * 3 + 1] * St[1][b] + V[i * 3 + 2] * St[2][b];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int i = I6[k][0], j = I6[k][1];
-    T acc = T(0);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) acc += V[i * 3 + a] * St[a][b] * V[j * 3 + b];
-    Pi[k] = acc;
+    Pi[k] = VS[i][0] * V[j * 3] + VS[i][1] * V[j * 3 + 1] + VS[i][2] * V[j * 3 + 2];
   }
   first_piola<T>(H, Pi, S);
 }
@@ -1047,15 +1109,18 @@ __device__ __forceinline__ void stress_sym(const ResParams<T>& P, int law, const
 // registers of the plain ones: held to four blocks (64 registers) the 128^3 J2 residual measured
 // k_stress 149 -> 112 us, k_stress_inc 144 -> 129, k_div 68 -> 52 / 81 -> 65; three blocks gave
 // 120 / 141 / 56 / 73, five (spills) 159 / 141 / 51 / 64.  FP64 is bound by its pipe and the
-// finite-strain laws by their own registers: no line for them.
+// logarithmic J2 by its own registers: no line for them; crystal plasticity in FP32 fits 128 registers.
 template <typename T, int SL>
-constexpr int resident_blocks() { return sizeof(T) == 4 && SL < 2 ? 4 : 0; }
+constexpr int resident_blocks() { return sizeof(T) == 4 && SL <= 2 ? (SL < 2 ? 4 : 2) : 0; }
 
 template <typename T, int TETRA, bool WITH_P, bool LO, bool SYM, int SL>
 __global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(ResParams<T> P, TileIdx ti) {
   if (P.stop && *P.stop) return;
   constexpr bool J2 = (SL & 1) != 0;
   constexpr int NPP = TETRA ? 2 : 1;
+  // crystal plasticity and logarithmic J2: a thread takes one point of its voxel (twice the threads
+  // to hide the laws' long chains with, and half the work left over in the last wave)
+  constexpr bool SPLIT = (SL & 6) && NPP == 2;
   constexpr int NC = SYM ? 6 : 9;
   constexpr int NCT = WITH_P ? NC + 9 : NC;
   __shared__ double red[32];
@@ -1065,9 +1130,9 @@ __global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(
   T sp = T(0);
   double SP = 0.0;
   int run = 0;
-  for (int t = blockIdx.x; t < ti.ntile; t += gridDim.x) {
+  for (int t = blockIdx.x; t < (SPLIT ? 2 : 1) * ti.ntile; t += gridDim.x) {
     int x0, y0, vz;
-    ti.at(t, &x0, &y0, &vz);
+    ti.at(SPLIT ? t >> 1 : t, &x0, &y0, &vz);
     const int vx = x0 + (threadIdx.x % RTX), vy_ = y0 + (threadIdx.x / RTX);
     if (vx < n1 && vy_ < n2) {
       T uh[3][8], ul[3][8];
@@ -1108,7 +1173,8 @@ __global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(
         stress_sym<T, TETRA, LO, J2>(P, law, lc, P.law_m + (size_t)ph * 36, j2, uh, ul, vx, vy_, vz, v, nvox, &spv);
       } else {
 #pragma unroll
-        for (int r = 0; r < NPP; ++r) {
+        for (int r0 = 0; r0 < (SPLIT ? 1 : NPP); ++r0) {
+          const int r = SPLIT ? t & 1 : r0;
           T Gf[9], Gt[9], Pp[9];
           law_grad<T, TETRA, LO>(P, j2, uh, ul, r, vx, vy_, vz, Gf, Gt);
           if (SL) point_law<T, SL>(P, law, lc, Gt, r, v, nvox, Pp, nullptr);
@@ -1984,7 +2050,8 @@ static int two_pass_blocks(const ResParams<T>& P) {
   TileIdx tn;
   FaceIdx fi;
   interior_and_faces<T>(P, &tn, &fi);
-  return std::max(std::min(RBLOCKS, tv.ntile), face_blocks<T>(fi) + std::min(RBLOCKS, std::max(1, tn.ntile)));
+  const int nv = (P.slaw & 6) ? 2 * tv.ntile : tv.ntile;  // k_stress's items: points, for those laws
+  return std::max(std::min(RBLOCKS, nv), face_blocks<T>(fi) + std::min(RBLOCKS, std::max(1, tn.ntile)));
 }
 
 template <typename T>
