@@ -1148,7 +1148,7 @@ int update_after(fftm_problem* p, int m, int cur0) {
       }
     }
     {
-      const int gb = gram_blocks(cnt);
+      const int gb = gram_blocks(sizeof(T) == 4 ? (cnt + 1) / 2 : cnt);  // FP32: two nodes a thread
       ProfScope ps(p, FFTM_KCAT_ANDERSON);
       CU(launch_gram<T>(Ds, depth, cnt, p->partial, gb, s, p->stop));
       if (p->stop)

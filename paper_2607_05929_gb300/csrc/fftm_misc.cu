@@ -94,7 +94,7 @@ cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, do
 }
 
 // The norms and the convergence test of Algorithm 1 on the device, in one launch (the sum of
-// the partials and the test were two: 10 + 4 us per iteration, now 5 with the same sums): err
+// the partials and the test were two: 10 + 4 us per iteration, now 5-8 with the same sums): err
 // (Eq. equilibrium_condition; +inf only means "not yet") is recorded at err_hist[m]; the step
 // stops when err < tol (1), on a non-finite norm (2) or at the iteration limit (3), else the
 // next iteration is m + 1.
@@ -158,7 +158,7 @@ cudaError_t launch_axpy_fields(T* const dst[3], const T* const a[3], const T* co
 }
 
 // Four blocks per SM, and no more than one element per thread needs: a block ends with 9 FP64
-// warp sums whatever it read (at 32^3 608 blocks took 22 us, 148 take 9).
+// warp sums whatever it read (at 32^3 608 blocks took 22 us, 148 take 16).
 int gram_blocks(long long count) { return (int)std::min<long long>(152 * 4, (count + 255) / 256); }
 
 // Normal matrix of the residual differences d_k = D_k - D_last (k < last) and
@@ -169,60 +169,71 @@ struct GramArgs {
   const T* D[4][3];
 };
 
-// Accumulator of a sum of products: FP64 for double data; for float data an
-// unevaluated pair (hi, lo) of floats updated with error-free transformations
-// (TwoProduct through fma, TwoSum), which keeps about twice FP32's precision
-// without the FP64 pipe (whose rate is a small fraction of FP32's on this GPU).
+// Accumulator of a sum of products: FP64 for double data; for float data an unevaluated pair
+// (hi, lo) of floats updated with error-free transformations (TwoProduct through fma, TwoSum),
+// which keeps about twice FP32's precision without the FP64 pipe (whose rate is a small fraction of
+// FP32's on this GPU).  Float data go two neighbouring nodes at a time in packed FP32x2
+// instructions, each with its own pair: ten instructions for two products.  256^3, four sets: 249 ->
+// 200 us (the reads alone 120); 128^3 58 -> 56.
 template <typename T>
-struct DotAcc {
+struct DotAcc;
+template <>
+struct DotAcc<double> {
+  using V = double;  // a thread's nodes of one step
   double s = 0.0;
-  __device__ __forceinline__ void add(T a, T b) { s += (double)a * (double)b; }
+  __device__ __forceinline__ void add(double a, double b) { s += a * b; }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
 struct DotAcc<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = a * b;
-    const float pe = fmaf(a, b, -p);  // exact error of the product
-    const float s = hi + p;
-    const float bb = s - hi;
-    const float se = (hi - (s - bb)) + (p - bb);  // exact error of the sum
-    hi = s;
-    lo += se + pe;
+  using V = float2;
+  float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+  static __device__ __forceinline__ float2 sub(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ void add(float2 a, float2 b) {
+    const float2 p = __fmul2_rn(a, b);
+    const float2 pe = __ffma2_rn(a, b, make_float2(-p.x, -p.y));  // exact error of the product
+    const float2 s = __fadd2_rn(hi, p);
+    const float2 bb = sub(s, hi);
+    const float2 se = __fadd2_rn(sub(hi, sub(s, bb)), sub(p, bb));  // exact error of the sum
+    hi = s;
+    lo = __fadd2_rn(lo, __fadd2_rn(se, pe));
+  }
+  __device__ __forceinline__ double value() const {
+    return ((double)hi.x + (double)lo.x) + ((double)hi.y + (double)lo.y);
+  }
 };
+__device__ __forceinline__ double v_sub(double a, double b) { return a - b; }
+__device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return DotAcc<float>::sub(a, b); }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_gram(GramArgs<T> A, int m, long long count, double* __restrict__ partial,
+// (four resident blocks: 64 registers of FP32 accumulators and loads; two to three blocks leave too
+// few loads in flight, 265 us, five spill, 421 us)
+template <typename T, int M>
+__global__ void __launch_bounds__(256, 4) k_gram(GramArgs<T> A, long long count, double* __restrict__ partial,
                                               const int* __restrict__ stop) {
   if (stop && *stop) return;
+  using V = typename DotAcc<T>::V;
+  constexpr int L = M - 1, W = sizeof(V) / sizeof(T);
   __shared__ double red[8][9];
   DotAcc<T> acc[9];
-  const int L = m - 1;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i * W < count;
        i += (long long)gridDim.x * blockDim.x) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      T v[4], d[3];
+      V v[M], d[3];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = (j < m) ? A.D[j][c][i] : T(0);
-      T last = v[0];
+      for (int j = 0; j < M; ++j) v[j] = reinterpret_cast<const V*>(A.D[j][c])[i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (j == L) last = v[j];
+      for (int j = 0; j < L; ++j) d[j] = v_sub(v[j], v[L]);
+      int k = 0;
 #pragma unroll
-      for (int j = 0; j < 3; ++j) d[j] = (j < L) ? v[j] - last : T(0);
-      acc[0].add(d[0], d[0]);
-      acc[1].add(d[0], d[1]);
-      acc[2].add(d[0], d[2]);
-      acc[3].add(d[1], d[1]);
-      acc[4].add(d[1], d[2]);
-      acc[5].add(d[2], d[2]);
-      acc[6].add(d[0], last);
-      acc[7].add(d[1], last);
-      acc[8].add(d[2], last);
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = a; b < 3; ++b, ++k)
+          if (b < L) acc[k].add(d[a], d[b]);
+#pragma unroll
+      for (int a = 0; a < L; ++a) acc[6 + a].add(d[a], v[L]);
     }
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -240,18 +251,23 @@ __global__ void __launch_bounds__(256) k_gram(GramArgs<T> A, int m, long long co
   }
 }
 
+// (a component, its padding included, is a multiple of 64 elements and starts at one: count is even
+// and pairs of nodes are aligned)
 template <typename T>
 cudaError_t launch_gram(const T* const D[4][3], int m, long long count, double* partial, int nblocks,
                         cudaStream_t s, const int* stop) {
   GramArgs<T> A;
   for (int j = 0; j < 4; ++j)
     for (int c = 0; c < 3; ++c) A.D[j][c] = (j < m) ? D[j][c] : D[0][c];
-  k_gram<T><<<nblocks, 256, 0, s>>>(A, m, count, partial, stop);
+  if (m <= 1) k_gram<T, 1><<<nblocks, 256, 0, s>>>(A, count, partial, stop);
+  else if (m == 2) k_gram<T, 2><<<nblocks, 256, 0, s>>>(A, count, partial, stop);
+  else if (m == 3) k_gram<T, 3><<<nblocks, 256, 0, s>>>(A, count, partial, stop);
+  else k_gram<T, 4><<<nblocks, 256, 0, s>>>(A, count, partial, stop);
   return cudaGetLastError();
 }
 
 // Reduce the partials (one warp per sum, its rows in flight together: a single warp that walked
-// them in a chain of dependent loads took 49-57 us at any grid size, this takes 6); solve
+// them in a chain of dependent loads took 49-57 us at any grid size, this takes 12-13); solve
 // (d^T d) gamma = -(d^T D_last) by Cholesky in FP64;
 // c_k = gamma_k (k < last), c_last = 1 - sum gamma.  A pivot below pivot_tol
 // times its diagonal entry rejects the step: c = e_last.

@@ -1485,7 +1485,7 @@ __device__ __forceinline__ T store_node(const ResParams<T>& P, int mx, int my, i
 // interior ones, where all 8 neighbouring voxels exist (or wrap): plain differences.  A face
 // node is a chain of index arithmetic and 24 gathers per component, bound by its latency, so
 // each thread takes one component of one node and the chains run beside the interior's
-// (43 -> 16 us at 32^3 in FP64, where a thread used to walk an interior node and then a face
+// (43 -> 19 us at 32^3 in FP64, where a thread used to walk an interior node and then a face
 // node with its three components in turn).
 template <typename T, int TETRA, bool WITH_P, bool SYM, bool INC>
 __global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0>()) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
@@ -1943,9 +1943,11 @@ __global__ void __launch_bounds__(FX * FY, 16 / FY) k_residual_fused(ResParams<T
 // layers that k_residual_fused stored; one S_D partial per block (S_P slot zero).  A thread
 // takes one component of one node (component-major, so that a warp walks one face): the
 // gathers of a node's three components run in parallel, and a component without a dof there
-// (every component of a fully Dirichlet face) writes its zero without any gather.
+// (every component of a fully Dirichlet face) writes its zero without any gather.  Bound by the
+// latency of the gathers: with four blocks of 256 an SM instead of two it takes 30 us at 192^3 (34)
+// and 43 at 256^3 (57); six and eight spill.
 template <typename T, int TETRA>
-__global__ void __launch_bounds__(256, 2) k_face_div(ResParams<T> P, FaceIdx fi) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_face_div(ResParams<T> P, FaceIdx fi) {
   if (P.stop && *P.stop) return;
   __shared__ double red[32];
   double SD = 0.0;
