@@ -913,7 +913,7 @@ __device__ __forceinline__ void cubic_strain(const double* __restrict__ m36, con
 // Small-strain elastic law of a phase at NP points (c: its law row; an isotropic phase keeps its
 // two constants, fewer products and roundings than the full stiffness).  One branch for the points
 // together: their products interleave and the stiffness is loaded once (the 192^3 FP32 one-pass
-// residual: 232 us, 248 with a branch per point).
+// residual: 226 us, 248 with a branch per point).
 template <typename T, int NP>
 __device__ __forceinline__ void elastic_strain(int law, const T* __restrict__ c, const T* __restrict__ m36,
                                                const T (&e)[NP][6], T (&p)[NP][6]) {
