@@ -1108,13 +1108,14 @@ __device__ __forceinline__ void stress_sym(const ResParams<T>& P, int law, const
 // its gathers, and its general paths (quadratic mean fields, face nodes) would otherwise set the
 // registers of the plain ones: held to four blocks (64 registers) the 128^3 J2 residual measured
 // k_stress 149 -> 112 us, k_stress_inc 144 -> 129, k_div 68 -> 52 / 81 -> 65; three blocks gave
-// 120 / 141 / 56 / 73, five (spills) 159 / 141 / 51 / 64.  FP64 is bound by its pipe and the
-// logarithmic J2 by its own registers: no line for them; crystal plasticity in FP32 fits 128 registers.
-template <typename T, int SL>
-constexpr int resident_blocks() { return sizeof(T) == 4 && SL <= 2 ? (SL < 2 ? 4 : 2) : 0; }
+// 120 / 141 / 56 / 73, five (spills) 159 / 141 / 51 / 64.  FP64 is bound by its pipe and
+// logarithmic J2 by its own registers: no line for them; crystal plasticity in FP32 fits 128
+// registers.  PLAIN: without the test outputs, and stresses of symmetric laws (the others would spill).
+template <typename T, int SL, bool PLAIN>
+constexpr int resident_blocks() { return sizeof(T) == 4 ? (SL < 2 ? (PLAIN ? 4 : 0) : (SL == 2 ? 2 : 0)) : 0; }
 
 template <typename T, int TETRA, bool WITH_P, bool LO, bool SYM, int SL>
-__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(ResParams<T> P, TileIdx ti) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL, SYM && !WITH_P>()) k_stress(ResParams<T> P, TileIdx ti) {
   if (P.stop && *P.stop) return;
   constexpr bool J2 = (SL & 1) != 0;
   constexpr int NPP = TETRA ? 2 : 1;
@@ -1235,7 +1236,7 @@ __global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, SL>()) k_stress(
 // P - P_n, with P_n the stress at the commit (elastic laws: the law applied to the
 // gradient increment; J2: j2_inc).  S_P still takes the full P.
 template <typename T, int TETRA, bool LO, bool SYM>
-__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0>()) k_stress_inc(ResParams<T> P, TileIdx ti) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0, SYM>()) k_stress_inc(ResParams<T> P, TileIdx ti) {
   if (P.stop && *P.stop) return;
   constexpr int NPP = TETRA ? 2 : 1;
   constexpr int NC = SYM ? 6 : 9;
@@ -1488,7 +1489,7 @@ __device__ __forceinline__ T store_node(const ResParams<T>& P, int mx, int my, i
 // (43 -> 19 us at 32^3 in FP64, where a thread used to walk an interior node and then a face
 // node with its three components in turn).
 template <typename T, int TETRA, bool WITH_P, bool SYM, bool INC>
-__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0>()) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
+__global__ void __launch_bounds__(RTX * RTY, resident_blocks<T, 0, !WITH_P>()) k_div(ResParams<T> P, TileIdx ti, FaceIdx fi, int nbf) {
   if (P.stop && *P.stop) return;
   constexpr int NC = SYM ? 6 : 9;
   constexpr int NCT = WITH_P ? NC + 9 : NC;
