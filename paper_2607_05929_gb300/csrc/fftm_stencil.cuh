@@ -796,17 +796,18 @@ __device__ __forceinline__ void law_grad(const ResParams<T>& P, bool j2, const T
 }
 
 // ---- small-strain laws straight from the stencil sums ------------------------------------
-// The differences of one displacement component along the three axes at a voxel point, from its
-// corner values (corner o = ox + 2 oy + 4 oz; sub and add in the field's arithmetic, packed
-// (hi, lo) pairs in FP32): the four-term sums of point_grad share their parts -- HEX1: the four
-// body diagonals' differences a, b, c, d give x = (a + b) + (c - d), y = (a + b) - (c - d),
-// z = (a - b) + (c + d), 11 operations for the three axes instead of 24; TETRA2: the tetrahedron's
-// four corners give x = A + B, y = A - B and z in 7 instead of 12.  Every term is still a
-// difference of neighbouring values.
-// The FP64 residual is bound by the FP64 pipe (two FMA a clock and SM), so these sums, the strain
-// and the divergence below in fewer operations are its time: 128^3 TETRA2 k_stress 778 -> 565 us,
-// k_div 355 -> 230 us.  FP32 issues fewer instructions (one pass, 192^3: 239 -> 226 us; 256^3 with
-// low parts 601 -> 519 us).
+// The sums of differences of one displacement component along the three axes at a voxel point, from
+// its corner values (corner o = ox + 2 oy + 4 oz; sub and add in the field's arithmetic, packed
+// (hi, lo) pairs in FP32): point_grad's differences, each along its own axis (HEX1) or the paper's
+// pair (TETRA2), added pairwise.  Sharing them between the axes (differences along the body
+// diagonals: 11 operations for three axes, 21 here; TETRA2 7, 9 here) makes a small derivative take
+// the rounding of a large one.  With these sums and the law and the divergence below, D in FP32 is
+// 0.974 to 0.997 times as far from 64 bits as by chains of additions on isotropic phases (shared
+// between the axes: 1.02 to 1.05 times), 0.96 to 0.985 times on cubic ones.
+// The strain, the law and the divergence take fewer operations than nine gradient components would:
+// FP64 is bound by its pipe (two FMA a clock and SM; 128^3 in two passes, cubic TETRA2 1229 -> 1013
+// us, isotropic HEX1 851 -> 678), FP32 issues fewer instructions (192^3 cubic TETRA2, one pass 290 ->
+// 269 us, two 353 -> 300).
 struct ScalarOps {
   template <typename V> static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
   template <typename V> static __device__ __forceinline__ V add(V a, V b) { return a + b; }
@@ -820,20 +821,15 @@ struct PairOps {  // FP32 (hi, lo), packed FP32x2 instructions
 
 template <typename Ops, int TETRA, typename V, typename U>
 __device__ __forceinline__ void corner_diffs(U&& u, int r, V s[3]) {
-  if constexpr (TETRA) {
-    // T1: corners 0 (000), 3 (110), 5 (101), 6 (011); T2: their opposites, whose differences along
-    // each axis are those of the point reflection
-    const V p = u(r == 0 ? 3 : 4), o = u(r == 0 ? 0 : 7), m = u(r == 0 ? 5 : 2), n = u(r == 0 ? 6 : 1);
-    const V A = r == 0 ? Ops::sub(p, o) : Ops::sub(o, p), B = r == 0 ? Ops::sub(m, n) : Ops::sub(n, m);
-    s[0] = Ops::add(A, B);
-    s[1] = Ops::sub(A, B);
-    s[2] = r == 0 ? Ops::add(Ops::sub(m, o), Ops::sub(n, p)) : Ops::add(Ops::sub(o, m), Ops::sub(p, n));
+  auto d = [&](int o1, int o0) { return Ops::sub(u(o1), u(o0)); };
+  if constexpr (TETRA) {  // T1: corners 0, 3, 5, 6; T2: 1, 2, 4, 7
+    s[0] = r == 0 ? Ops::add(d(3, 0), d(5, 6)) : Ops::add(d(1, 2), d(7, 4));
+    s[1] = r == 0 ? Ops::add(d(6, 0), d(3, 5)) : Ops::add(d(7, 1), d(2, 4));
+    s[2] = r == 0 ? Ops::add(d(5, 0), d(6, 3)) : Ops::add(d(4, 1), d(7, 2));
   } else {
-    const V a = Ops::sub(u(7), u(0)), b = Ops::sub(u(3), u(4)), c = Ops::sub(u(5), u(2)), d = Ops::sub(u(6), u(1));
-    const V ab = Ops::add(a, b), cd = Ops::sub(c, d);
-    s[0] = Ops::add(ab, cd);
-    s[1] = Ops::sub(ab, cd);
-    s[2] = Ops::add(Ops::sub(a, b), Ops::add(c, d));
+    s[0] = Ops::add(Ops::add(d(1, 0), d(3, 2)), Ops::add(d(5, 4), d(7, 6)));
+    s[1] = Ops::add(Ops::add(d(2, 0), d(3, 1)), Ops::add(d(6, 4), d(7, 5)));
+    s[2] = Ops::add(Ops::add(d(4, 0), d(5, 1)), Ops::add(d(6, 2), d(7, 3)));
   }
 }
 
@@ -913,7 +909,9 @@ __device__ __forceinline__ void cubic_strain(const double* __restrict__ m36, con
 // Small-strain elastic law of a phase at NP points (c: its law row; an isotropic phase keeps its
 // two constants, fewer products and roundings than the full stiffness).  One branch for the points
 // together: their products interleave and the stiffness is loaded once (the 192^3 FP32 one-pass
-// residual: 226 us, 248 with a branch per point).
+// residual: 226 us, 248 with a branch per point).  The trace's share enters its FMA unrounded: a
+// small normal stress beside a large one would else take the rounding of that one's share (D beside
+// a face that the field is cut to zero at: 1.03 to 1.08 times as far from 64 bits).
 template <typename T, int NP>
 __device__ __forceinline__ void elastic_strain(int law, const T* __restrict__ c, const T* __restrict__ m36,
                                                const T (&e)[NP][6], T (&p)[NP][6]) {
@@ -924,9 +922,9 @@ __device__ __forceinline__ void elastic_strain(int law, const T* __restrict__ c,
     const T lam = __ldg(c), mu = __ldg(c + 1), mu2 = T(2) * mu;
 #pragma unroll
     for (int r = 0; r < NP; ++r) {
-      const T tr = lam * ((e[r][0] + e[r][1]) + e[r][2]);
+      const T tr = (e[r][0] + e[r][1]) + e[r][2];
 #pragma unroll
-      for (int a = 0; a < 6; ++a) p[r][a] = a < 3 ? fma(mu2, e[r][a], tr) : mu * e[r][a];
+      for (int a = 0; a < 6; ++a) p[r][a] = a < 3 ? fma(lam, tr, mu2 * e[r][a]) : mu * e[r][a];
     }
   }
 }
@@ -943,19 +941,18 @@ __device__ __forceinline__ T norm6(const T p[6]) {  // |P|^2
 // voxel point on corner o: the sums over the corners along axis i, sum over pairs of differences.
 // A shear component is differenced along two axes i, j: the differences along the face diagonals,
 // A = sum (v_11 - v_00) and B = sum (v_10 - v_01), give A + B and A - B: 54 operations for the
-// three components of D instead of 81.
+// three components of D instead of 81 (FP64 128^3 in two passes: 9 % of the residual).  Each sum then
+// takes the rounding of the other axis' variation, of the size of the rounding that the stresses
+// bring along; added pairwise and in the order of the axes D is nearer to 64 bits all the same than
+// by chains of differences along each axis (figures at corner_diffs).
 template <typename T, typename V>
 __device__ __forceinline__ void sym_div(V&& v, const T* w, T D[3]) {
+  T s[3][3];  // along axis i, of component (i, q)
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    T s = T(0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int lowbits = (1 << i) - 1, o = ((k & ~lowbits) << 1) | (k & lowbits);  // corners with o_i = 0
-      const T d = v(i, o | (1 << i)) - v(i, o);
-      s = k == 0 ? d : s + d;
-    }
-    D[i] = w[i] * s;
+    const int b = 1 << i, k = i == 0 ? 2 : 1, l = i == 2 ? 2 : 4;  // the axis and the two others
+    auto d = [&](int o) { return v(i, o | b) - v(i, o); };
+    s[i][i] = (d(0) + d(k)) + (d(l) + d(k | l));
   }
 #pragma unroll
   for (int c = 3; c < 6; ++c) {
@@ -963,9 +960,11 @@ __device__ __forceinline__ void sym_div(V&& v, const T* w, T D[3]) {
     const int bi = 1 << i, bj = 1 << j, bm = 1 << m;
     const T A = (v(c, bi | bj) - v(c, 0)) + (v(c, bi | bj | bm) - v(c, bm));
     const T B = (v(c, bi) - v(c, bj)) + (v(c, bi | bm) - v(c, bj | bm));
-    D[j] = fma(w[i], A + B, D[j]);
-    D[i] = fma(w[j], A - B, D[i]);
+    s[i][j] = A + B;
+    s[j][i] = A - B;
   }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) D[q] = fma(w[2], s[2][q], fma(w[1], s[1][q], w[0] * s[0][q]));
 }
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
