@@ -4,14 +4,23 @@ plan tests' tolerances leave room for (angles of the tables rounded before the c
 FP64: an FFT of N points with tables good to a unit rounds by about 0.6 u sqrt(log2 N) relative to
 its result, u = 2^-53 (Schatzman 1996, the average case); the pre- and post-processing add about one
 such step to the log2 N, and the bound is u sqrt(log2 N), five thirds of the average.  The sums are
-formed in long double from angles reduced in integers."""
+formed in long double from angles reduced in integers.
+
+FP32: roundings are unbiased, a constant that is off its FP32 value is not: it scales what it
+multiplies.  Of a DFT of 256 points (two stages of radix 16) the spectrum's mean scale must not be off
+by more than sqrt(1/2) alone explains, 1.7e-8 from its FP32 value on a quarter of the elements of each
+stage: 0.85e-8; the 225 table entries, rounded independently, add 3e-8 / 15 = 2e-9, and the average
+over 49152 outputs leaves 6e-10 of their roundings (one standard deviation each).  The bound, 2e-8, is
+that plus five times both deviations."""
 
 import numpy as np
 import pytest
 
+from abi_helpers import GpuProblem, oracle_r2r_forward
 from oracle.bc import dof_range
 from paper_2607_05929_gb300 import build
 from paper_2607_05929_gb300 import fftm as F
+from synthetic.workloads import ISO_ELASTIC, Material, Workload, axis_bc
 
 pytestmark = pytest.mark.gpu
 
@@ -60,3 +69,24 @@ def test_fp64_transforms_round_like_an_fft_with_exact_tables(kind, n):
     bound = 2.0 ** -53 * np.sqrt(np.log2(n))
     for name, (e2, r2) in err.items():
         assert np.sqrt(e2 / r2) <= bound, (name, np.sqrt(e2 / r2), bound)
+
+
+def test_fp32_radix_16_stages_do_not_scale_the_spectrum():
+    n = (256, 2, 2)
+    wl = Workload("dft", n, np.zeros(n, dtype=np.int32), [Material(ISO_ELASTIC, (1.0, 1.0))],
+                  axis_bc("P", "P", "P"), scheme="HEX1", lambda0=1.0, mu0=1.0)
+    gp = GpuProblem(wl, "fp32")
+    num = den = 0.0
+    try:
+        for seed in range(16):
+            x = np.random.default_rng(seed).standard_normal((3,) + n).astype(np.float32).astype(np.float64)
+            gp.set_node(F.FFTM_FIELD_WORK, x)
+            F.fftm_apply(gp.p, F.FFTM_OP_DT_FORWARD)
+            X = gp.get_node(F.FFTM_FIELD_WORK)
+            for q in range(3):
+                ref = oracle_r2r_forward(x[q], ["DFT"] * 3, n, n)
+                num += float(np.vdot(X[q] - ref, ref))
+                den += float(np.vdot(ref, ref))
+    finally:
+        gp.close()
+    assert abs(num / den) <= 2e-8, num / den
