@@ -2354,22 +2354,32 @@ cudaError_t launch_voxel_fields(const ResParams<T>& P, int tetra, T* grad_out, T
 }
 
 // ---- volume means of P and G (step report, normal-mixed loading) ----
-// A sum of field values that keeps FP64's precision: FP64 adds for double data; for float data an
-// unevaluated pair of floats updated with TwoSum (this GPU's FP64 pipe takes a conversion or an
-// add of one warp every 16 cycles, so 18 sums in FP64 cost more than the law they sum).
+// A sum of field values with FP64's precision: FP64 adds for double data; for float data an
+// unevaluated sum of three floats, the first two updated with TwoSum (72 bits; this GPU's FP64 pipe
+// takes a conversion or an add of one warp every 16 cycles, so that 18 sums in FP64 cost more than the
+// law they sum; two floats, 48 bits, drop what an FP64 sum of 53 keeps).  A sum that is not finite is
+// its first part, as in FP64.  256^3 TETRA2, one residual and these sums: 1.38 ms (two floats 1.28,
+// FP64 sums 3.97 with the instances of every law in one).
 template <typename T>
-struct SumAcc {
-  T hi = T(0), lo = T(0);
-  __device__ __forceinline__ void add(T a) {
-    if constexpr (sizeof(T) == 8) {
-      hi += a;
-    } else {
-      const T s = hi + a, b = s - hi;
-      lo += (hi - (s - b)) + (a - b);
-      hi = s;
-    }
+struct SumAcc;
+template <>
+struct SumAcc<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a) { s += a; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct SumAcc<float> {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
+  static __device__ __forceinline__ float two_sum(float* s, float a) {  // *s += a; the exact error
+    const float t = *s + a, b = t - *s, e = (*s - (t - b)) + (a - b);
+    *s = t;
+    return e;
   }
-  __device__ __forceinline__ double value() const { return sizeof(T) == 8 ? (double)hi : (double)hi + (double)lo; }
+  __device__ __forceinline__ void add(float a) { lo += two_sum(&mid, two_sum(&hi, a)); }
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+  }
 };
 
 // Sums of NV accumulators over the block -> row[0 .. NV): one value per warp at a time from
