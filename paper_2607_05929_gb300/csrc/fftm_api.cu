@@ -783,11 +783,16 @@ std::mutex g_tune_mu;
 std::map<std::string, std::string> g_tune_table;  // key -> "choice (times)"
 std::map<std::string, int> g_tune_choice;
 
+// What a choice depends on: the grid's shape, the law (one for all phases or read per voxel: the
+// kernels branch on it), and the forms compared -- a problem that asks for one pass compares its tiles
+// alone, and what it finds says nothing about two passes.
 std::string residual_key(const fftm_problem* p) {
-  char b[160];
-  std::snprintf(b, sizeof(b), "residual %s %s %dx%dx%d %c%c%c", p->esz == 8 ? "fp64" : "fp32",
+  char law[8] = "mixed";
+  if (p->one_law >= 0) std::snprintf(law, sizeof(law), "law %d", p->one_law);
+  char b[192];
+  std::snprintf(b, sizeof(b), "residual %s %s %dx%dx%d %c%c%c %s%s", p->esz == 8 ? "fp64" : "fp32",
                 p->tetra ? "TETRA2" : "HEX1", p->n[0], p->n[1], p->n[2], p->periodic[0] ? 'P' : 'B',
-                p->periodic[1] ? 'P' : 'B', p->periodic[2] ? 'P' : 'B');
+                p->periodic[1] ? 'P' : 'B', p->periodic[2] ? 'P' : 'B', law, p->res_passes == 1 ? " one pass" : "");
   return b;
 }
 
@@ -841,7 +846,7 @@ int resolve_residual_form(fftm_problem* p, int slot) {
     auto it = g_tune_choice.find(key);
     if (it != g_tune_choice.end()) {
       const int c = it->second;  // 0: one pass, fy 8; 1: one pass, fy 16; 2: two passes
-      p->res_two_pass = (p->res_passes == 1) ? 0 : (c == 2 ? 1 : 0);
+      p->res_two_pass = c == 2 ? 1 : 0;
       p->res_fy = c == 1 ? 16 : 8;
       return FFTM_OK;
     }
@@ -855,8 +860,9 @@ int resolve_residual_form(fftm_problem* p, int slot) {
   if (t2 >= 0.0 && (best < 0.0 || t2 < best)) c = 2, best = t2;
   static const char* names[3] = {"one pass, 8-row tiles", "one pass, 16-row tiles", "two passes"};
   char b[200];
-  std::snprintf(b, sizeof(b), "%s (one pass 8 rows %.4f ms, 16 rows %.4f ms; two passes %.4f ms)", names[c], t8, t16,
-                t2);
+  int len = std::snprintf(b, sizeof(b), "%s (one pass 8 rows %.4f ms, 16 rows %.4f ms", names[c], t8, t16);
+  if (p->res_passes != 1) len += std::snprintf(b + len, sizeof(b) - len, "; two passes %.4f ms", t2);
+  std::snprintf(b + len, sizeof(b) - len, ")");
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_choice[key] = c;
