@@ -439,10 +439,13 @@ int fftm_kernel_times(const fftm_problem* p, double* ms, long long* launches, in
    Asynchronous: results are ready when the problem's stream reaches them.
    Scratch: the reduction's block partials live in a file-scope device array
    of 16384 doubles (128 KiB) that every GPU loading the library holds until
-   the process exits (the residual kernels use a few thousand blocks at
-   most, whatever the grid, 2 slots each; a launch needing more than 16380 slots would be rejected with
-   FFTM_E_UNSUPPORTED and a message); the voxel-point stresses go to a buffer
-   the problem allocated when it was created.  Every slot read is written earlier in the same call, so nothing
+   the process exits, 2 slots a block of the residual kernels; a launch that
+   needs more is rejected with FFTM_E_UNSUPPORTED and a message.  The two-pass
+   kernels take at most 3648 blocks.  The one-pass kernel takes up to 4000 and
+   one more per tile of 31 x 7 nodes of a z plane, 1216 more with non-periodic
+   axes: planes of 768 x 768 always fit, a periodic 1536 x 1536 grid (11000
+   tiles) does not.  The voxel-point stresses go to a buffer the
+   problem allocated when it was created.  Every slot read is written earlier in the same call, so nothing
    needs clearing; all calls share the array, so calls that overlap on the GPU
    (other streams, other threads, other problems on the same device) race.
    The first call on a device looks the array's device address up

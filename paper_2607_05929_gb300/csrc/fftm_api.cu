@@ -1659,7 +1659,7 @@ Sizes sizes_of(const fftm_problem_desc* d) {
   size_t t = 0;
   for (int a = 0; a < 3; ++a) {
     const int M = 2 * d->n[a] + 2;
-    t += 3 * ((size_t)M * 2 + 16 + (size_t)M * 2 * esz + 16 + (size_t)(d->n[a] + 2) * 2 * esz + 16 +
+    t += 3 * ((size_t)M * 2 * esz + 16 + (size_t)(d->n[a] + 2) * 2 * esz + 16 +
               2 * ((size_t)(d->n[a] + 2) * esz + 16));
   }
   s.tables = t + 4096;
@@ -2752,7 +2752,7 @@ int fftm_kernel_launches(const fftm_problem* p, long long* count) {
 // GPU, held until the process exits).
 namespace {
 
-constexpr int kNoAllocScratchDoubles = 16384;  // 128 KiB of block partials + 4 result slots
+constexpr int kNoAllocScratchDoubles = 16384;  // 128 KiB of block partials
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];
 
 constexpr int kMaxDevices = 64;
@@ -2792,11 +2792,11 @@ int residual_noalloc_t(fftm_problem* p, const T* u, T* D, double* norms) {
   R.sy = p->N[0];
   R.sz = (long long)p->N[0] * p->N[1];
   const int blocks = residual_blocks<T>(R, p->tetra);
-  if (2LL * blocks > kNoAllocScratchDoubles - 4)
+  if (2LL * blocks > kNoAllocScratchDoubles)
     return set_err(FFTM_E_UNSUPPORTED, "grid too large for the no-allocation scratch (" +
                                            std::to_string(blocks) + " blocks need " + std::to_string(2 * blocks) +
                                            " doubles; the maximum is " +
-                                           std::to_string(kNoAllocScratchDoubles - 4) + ")");
+                                           std::to_string(kNoAllocScratchDoubles) + ")");
   R.partial = scratch;  // every block overwrites its two slots: nothing has to start at zero
   cudaStream_t s = p->ctx->stream;
   CU(launch_residual<T>(R, p->tetra, false, s, nullptr));

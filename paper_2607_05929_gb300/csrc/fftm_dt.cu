@@ -442,18 +442,15 @@ __device__ __forceinline__ void pre_item(const AxisPlan<T>& pl, bool inverse, in
   }
 }
 
-// The kinds whose items load one row each (DFT forward, DCT-II, DST-II): their loads are issued
-// PRE_BATCH items at a time, since one load per trip leaves a pass waiting for memory.
-__device__ __forceinline__ bool pre_single(int kind, bool inverse) {
+// DFT forward, DCT-II and DST-II: an item of the pre-processing loads one row (the loads are issued
+// PRE_BATCH items at a time, since one load per trip leaves a pass waiting for memory), and the outputs
+// pair the FFT bins k and n - k: items 0 .. n / 2 of post_item, each the rows r0 and r1 (r1 < 0: only
+// the first).
+__device__ __forceinline__ bool rows_in_pairs_out(int kind, bool inverse) {
   return kind == K_DFT ? !inverse : (inverse && (kind == K_DCT3 || kind == K_DST3));
 }
 constexpr int PRE_BATCH = 8;
 
-// Whether a transform's outputs pair the FFT bins k and n - k (DFT forward, DCT-II, DST-II):
-// items 0 .. n / 2 of post_item, each the rows r0 and r1 (r1 < 0: only the first).
-__device__ __forceinline__ bool paired_outputs(int kind, bool inverse) {
-  return kind == K_DFT ? !inverse : (inverse && (kind == K_DCT3 || kind == K_DST3));
-}
 template <typename T, int SP>
 __device__ __forceinline__ void post_item(const AxisPlan<T>& pl, const v2<T>* z, int k, int* r0, v2<T>* o0, int* r1,
                                           v2<T>* o1) {
@@ -591,7 +588,7 @@ __global__ void __launch_bounds__(pass_threads<T, FUSED>(), pass_ctas<T, FUSED>(
     const int items = pre_items(pl, inv_first);
     if (AXIS == 0) {
       RowItems f(items);
-      if (pre_single(pl.kind, inv_first)) {
+      if (rows_in_pairs_out(pl.kind, inv_first)) {
         while (f.p < W) {
           v2<T> v[PRE_BATCH];
           int fp[PRE_BATCH], fi[PRE_BATCH];
@@ -626,7 +623,7 @@ __global__ void __launch_bounds__(pass_threads<T, FUSED>(), pass_ctas<T, FUSED>(
         return v;
       };
       auto st = [&](int m, const v2<T>& v) { buf0[m * SP + pc] = v; };
-      if (pre_single(pl.kind, inv_first)) {
+      if (rows_in_pairs_out(pl.kind, inv_first)) {
         for (int i = i0; i < items; i += PRE_BATCH * istep) {
           v2<T> v[PRE_BATCH];
 #pragma unroll
@@ -693,7 +690,7 @@ __global__ void __launch_bounds__(pass_threads<T, FUSED>(), pass_ctas<T, FUSED>(
 
   // ---- results -> global ----
   const T sc = P.scale[q];
-  const bool paired = paired_outputs(pl.kind, inverse);
+  const bool paired = rows_in_pairs_out(pl.kind, inverse);
   const int items = paired ? pl.n / 2 + 1 : L;
   if (AXIS != 0) {
     const v2<T>* z = buf(cur) + pc;

@@ -286,8 +286,7 @@ template <typename T>
 cudaError_t launch_state_io(const ResParams<T>& P, int tetra, T* out, const T* in, cudaStream_t s);
 
 // out[v] = sum over the rows of partial[row * nvals + v]
-cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
-                               const int* stop = nullptr);
+cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s);
 // S_D and S_P of the residual's block partials (rows of two, 16-byte aligned) -> sums[0..1] and,
 // with err_too, err = h1 sqrt(S_D / S_P) -> sums[2]
 cudaError_t launch_norms(const double* partial, int nblocks, double* sums, bool err_too, double h1, cudaStream_t s,
@@ -334,30 +333,13 @@ int gram_blocks(long long count);
 // Measured FMA throughput of the current device (FLOP/s, an FMA counting two), FP64 or FP32.
 double fma_peak_flops(int fp64);
 
-// Asynchronous global -> shared copies (cp.async, Ampere and later): the copy
-// is issued without a register round trip, so a thread can keep many loads in
-// flight; cp_async_wait_all() + __syncthreads() make them visible.
-__device__ __forceinline__ void cp_async_4(void* smem, const void* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_8(void* smem, const void* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
-  if (sizeof(T) == 8) cp_async_8(smem, gmem);
-  else cp_async_4(smem, gmem);
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-// wait until at most one committed group is still in flight
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+
 // Sums over the voxel points: rows of 18 (P[3 i + q], then G[3 i + q]), their count in *nblocks.
 template <typename T>
 cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s);
-// The same for P alone (rows of 9), from the stresses that a plain two-pass residual left in P.vs.
+// The same for P alone (rows of 9), from the symmetric stresses that a plain two-pass residual left in
+// P.vs.
 template <typename T>
 cudaError_t launch_stress_sums(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s);
 

@@ -23,9 +23,7 @@ namespace fftm {
 // Sum `nvals` doubles over `nblocks` rows (fixed order: deterministic).  One warp per column:
 // FP64 adds issue at one warp instruction in 16 cycles per SM here, so the sums are arranged
 // for few of them (a lane's rows, then five shuffles per column).
-__global__ void k_reduce(const double* __restrict__ partial, int nblocks, int nvals, double* __restrict__ out,
-                         const int* __restrict__ stop) {
-  if (stop && *stop) return;
+__global__ void k_reduce(const double* __restrict__ partial, int nblocks, int nvals, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   for (int v = threadIdx.x >> 5; v < nvals; v += blockDim.x >> 5) {
     double s = 0.0;
@@ -87,9 +85,8 @@ cudaError_t launch_norms(const double* partial, int nblocks, double* sums, bool 
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s,
-                               const int* stop) {
-  k_reduce<<<1, 32 * (nvals < 32 ? nvals : 32), 0, s>>>(partial, nblocks, nvals, out, stop);
+cudaError_t launch_reduce_sums(const double* partial, int nblocks, int nvals, double* out, cudaStream_t s) {
+  k_reduce<<<1, 32 * (nvals < 32 ? nvals : 32), 0, s>>>(partial, nblocks, nvals, out);
   return cudaGetLastError();
 }
 

@@ -31,8 +31,9 @@
 // (-1 if i is the face normal) on component (i, q), and with T1 <-> T2
 // swapped once per face crossed (Sec. 2.2, Sec. 2.5.2).  Periodic axes wrap.
 #pragma once
-// Included by fftm_stencil_f32.cu and fftm_stencil_f64.cu, which instantiate the launchers for
-// one precision each (two translation units that compile in parallel).
+// Included by fftm_stencil_f32.cu and fftm_stencil_f64.cu, which instantiate the residual's launchers
+// for one precision each, and by fftm_fields_f32.cu and fftm_fields_f64.cu, which do so for the commit,
+// state, field and statistics kernels (four translation units that compile in parallel).
 #include <algorithm>
 
 #include "fftm_internal.cuh"
@@ -2445,47 +2446,37 @@ cudaError_t launch_stats(const ResParams<T>& P, int tetra, double* partial, int*
 }
 
 // The sum of P alone, from the voxel-point stresses that the two-pass residual has just stored
-// (its plain form): normal-mixed loading needs the mean stress after every residual, and
-// evaluating every point's law again for it cost as much as the residual's own k_stress
-// (103 us an iteration of a 64^3 FP64 problem).
-template <typename T, int NPP, bool SYM>
+// (its plain form; normal-mixed loads take small-strain laws alone, symmetric P): the mean stress is
+// needed after every residual, and evaluating every point's law again for it cost as much as the
+// residual's own k_stress (103 us an iteration of a 64^3 FP64 problem).
+template <typename T, int NPP>
 __global__ void __launch_bounds__(RTX * RTY) k_stress_sums(const T* __restrict__ vs, long long nvox,
                                                            double* __restrict__ partial) {
-  constexpr int NC = SYM ? 6 : 9;
-  SumAcc<T> acc[9];
+  SumAcc<T> sum[6];  // 11, 22, 33, 23, 13, 12
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox;
        v += (long long)gridDim.x * blockDim.x) {
-    T p[NPP][NC];
+    T p[NPP][6];
 #pragma unroll
     for (int r = 0; r < NPP; ++r)
 #pragma unroll
-      for (int c = 0; c < NC; ++c) p[r][c] = __ldg(vs + (size_t)(r * NC + c) * nvox + v);
+      for (int c = 0; c < 6; ++c) p[r][c] = __ldg(vs + (size_t)(r * 6 + c) * nvox + v);
 #pragma unroll
     for (int r = 0; r < NPP; ++r)
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c].add(p[r][c]);
+      for (int c = 0; c < 6; ++c) sum[c].add(p[r][c]);
   }
-  if (SYM) {  // (11, 22, 33, 23, 13, 12) -> P[3 i + q]
-    const SumAcc<T> a0 = acc[0], a1 = acc[1], a2 = acc[2], a3 = acc[3], a4 = acc[4], a5 = acc[5];
-    acc[0] = a0; acc[1] = a5; acc[2] = a4;
-    acc[3] = a5; acc[4] = a1; acc[5] = a3;
-    acc[6] = a4; acc[7] = a3; acc[8] = a2;
-  }
+  const SumAcc<T> acc[9] = {sum[0], sum[5], sum[4], sum[5], sum[1], sum[3], sum[4], sum[3], sum[2]};  // P[3 i + q]
   block_sums<T, 9>(acc, partial + (size_t)blockIdx.x * 9);
 }
 
 template <typename T>
 cudaError_t launch_stress_sums(const ResParams<T>& P, int tetra, double* partial, int* nblocks, cudaStream_t s) {
+  if (!P.sym) return cudaErrorInvalidValue;
   const long long nvox = (long long)P.n[0] * P.n[1] * P.n[2];
   const int nb = (int)std::min<long long>(STATS_BLOCKS, (nvox + RTX * RTY - 1) / (RTX * RTY));
   *nblocks = nb;
-  if (tetra) {
-    if (P.sym) k_stress_sums<T, 2, true><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
-    else k_stress_sums<T, 2, false><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
-  } else {
-    if (P.sym) k_stress_sums<T, 1, true><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
-    else k_stress_sums<T, 1, false><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
-  }
+  if (tetra) k_stress_sums<T, 2><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
+  else k_stress_sums<T, 1><<<nb, RTX * RTY, 0, s>>>(P.vs, nvox, partial);
   return cudaGetLastError();
 }
 
