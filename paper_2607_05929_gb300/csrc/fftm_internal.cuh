@@ -47,6 +47,10 @@ struct AxisPlan {
 template <typename T>
 struct PassParams {
   const T* in[3];
+  // Zero on entry at every position that the component does not transform along some axis (its
+  // dismissed nodes): a pass leaves those as they are.  Every writer of the problem's fields keeps
+  // them zero: cleared at creation and on reset, masked where a caller's field comes in, written as
+  // zeros by the residual, combined only with themselves.
   T* out[3];
   // optional accumulation at store (last inverse pass of the solver update):
   // out = base + scale * value, as an unevaluated hi + lo pair when out_lo is set

@@ -204,8 +204,9 @@ struct DotAcc<float> {
 __device__ __forceinline__ double v_sub(double a, double b) { return a - b; }
 __device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return DotAcc<float>::sub(a, b); }
 
-// (four resident blocks: 64 registers of FP32 accumulators and loads; two to three blocks leave too
-// few loads in flight, 265 us, five spill, 421 us)
+// (four resident blocks: 64 registers of FP32 accumulators and loads, of which the instance for four
+// sets spills 132 bytes a thread; two to three blocks leave too few loads in flight, 265 us, five spill
+// more, 421 us)
 template <typename T, int M>
 __global__ void __launch_bounds__(256, 4) k_gram(GramArgs<T> A, long long count, double* __restrict__ partial,
                                               const int* __restrict__ stop) {

@@ -1108,9 +1108,14 @@ __device__ __forceinline__ void stress_sym(const ResParams<T>& P, int law, const
 // its gathers, and its general paths (quadratic mean fields, face nodes) would otherwise set the
 // registers of the plain ones: held to four blocks (64 registers) the 128^3 J2 residual measured
 // k_stress 149 -> 112 us, k_stress_inc 144 -> 129, k_div 68 -> 52 / 81 -> 65; three blocks gave
-// 120 / 141 / 56 / 73, five (spills) 159 / 141 / 51 / 64.  FP64 is bound by its pipe and
-// logarithmic J2 by its own registers: no line for them; crystal plasticity in FP32 fits 128
-// registers.  PLAIN: without the test outputs, and stresses of symmetric laws (the others would spill).
+// 120 / 141 / 56 / 73, five 159 / 141 / 51 / 64.  The hidden latency is worth more than the spills
+// that four blocks cost (with low parts all 48 corner values of a voxel are alive at once:
+// k_stress_inc stores 440-456 bytes a thread, k_stress with J2 196, k_div's face nodes 40).  The
+// divergence of nine-component stresses (finite strain) gains too: the 128^3 residual of
+// St-Venant-Kirchhoff phases 130 -> 117 us HEX1, 158 -> 146 TETRA2, neo-Hookean 132 -> 120, 164 -> 150.
+// FP64 is bound by its pipe and logarithmic J2 by its own registers: no line for them; crystal
+// plasticity in FP32 fits 128 registers.  PLAIN: without the test outputs and, for the stress kernels,
+// of symmetric laws (the others were not measured under the line).
 template <typename T, int SL, bool PLAIN>
 constexpr int resident_blocks() { return sizeof(T) == 4 ? (SL < 2 ? (PLAIN ? 4 : 0) : (SL == 2 ? 2 : 0)) : 0; }
 
@@ -1946,7 +1951,8 @@ __global__ void __launch_bounds__(FX * FY, 16 / FY) k_residual_fused(ResParams<T
 // gathers of a node's three components run in parallel, and a component without a dof there
 // (every component of a fully Dirichlet face) writes its zero without any gather.  Bound by the
 // latency of the gathers: with four blocks of 256 an SM instead of two it takes 30 us at 192^3 (34)
-// and 43 at 256^3 (57); six and eight spill.
+// and 43 at 256^3 (57) although 40 bytes a thread spill; six and eight spill more and take as long as
+// two (46 and 55 at 256^3).
 template <typename T, int TETRA>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_face_div(ResParams<T> P, FaceIdx fi) {
   if (P.stop && *P.stop) return;
