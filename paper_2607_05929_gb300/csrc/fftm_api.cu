@@ -119,17 +119,18 @@ bool factor_stages(int N, int S, int* rad) {
 }
 
 // (c, s) = (cos, sin) of 2 pi t / n, t >= 0, good to a unit: the angle is reduced to at most pi / 4 in
-// integers and held in long double.  An angle of up to 2 pi rounded to FP64 first is off by up to four
+// integers and held in two parts.  An angle of up to 2 pi rounded to FP64 first is off by up to four
 // units of its cosine; the FP64 transforms then took up to half of their error from these tables, and
 // those of 24 and 216 points, whose two or three stages meet more of the large angles than stages of 3
 // and 8 do, came out further from the exact sums than with those (by 4 and 11 %).
 void unit_root(long long t, long long n, double* c, double* s) {
-  const long double quarter = 1.57079632679489661923132169163975144L;
+  const double quarter = 1.57079632679489661923, quarter_lo = 6.123233995736766036e-17;  // pi / 2
   t %= n;
   const long long q = 4 * t / n, r = 4 * t % n;  // q quarter turns and r / n of one
   const bool far = 2 * r > n;
-  const long double a = quarter * (long double)(far ? n - r : r) / (long double)n;
-  const double x = (double)std::cos(a), y = (double)std::sin(a);
+  const double m = (double)(far ? n - r : r), f = m / (double)n, f_lo = std::fma(-f, (double)n, m) / (double)n;
+  const double a = quarter * f, a_lo = std::fma(quarter, f, -a) + (quarter_lo * f + quarter * f_lo);
+  const double ca = std::cos(a), sa = std::sin(a), x = ca - a_lo * sa, y = sa + a_lo * ca;
   const double u = far ? y : x, v = far ? x : y;
   *c = q == 0 ? u : (q == 1 ? -v : (q == 2 ? -u : v));
   *s = q == 0 ? v : (q == 1 ? u : (q == 2 ? -v : -u));
