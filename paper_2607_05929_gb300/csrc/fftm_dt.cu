@@ -24,7 +24,7 @@
 // addition per element and level.  FP64 data: the FP64 pipe bounds the pass, and half of the FFT's
 // work goes (128^3: x 415 -> 225 us, y 385 -> 220, fused z 821 -> 436).  FP32 data: instruction
 // issue and latency bound it, and the passes through shared memory and their barriers go (256^3: x
-// 319 -> 230 us, y 352 -> 189, fused z 627 -> 222; the copy rate would allow 60).
+// 319 -> 230 us, y 352 -> 193, fused z 627 -> 221; the copy rate would allow 60).
 //
 // The fused z pass multiplies the z spectrum by the Green factor (Eqs.
 // NSGO1_*, NSGO2_*) and runs the inverse z transform without leaving the SM.
@@ -499,8 +499,8 @@ __device__ __forceinline__ GreenLine<T> green_line(const PassParams<T>& P, int q
 }
 
 // Threads per CTA at most.  FP32 type-I passes along x and y have two CTAs an SM at 256 voxels
-// (82 KB of buffers): 512 threads each (x 263 -> 230 us, y 208 -> 189); the fused z pass has three
-// (z 238 us with 512, 222 with 256).
+// (82 KB of buffers): 512 threads each (x 263 -> 230 us, y 208 -> 193); the fused z pass has three
+// (z 238 us with 512, 221 with 256).
 template <typename T, int FUSED>
 constexpr int pass_threads() { return sizeof(T) == 4 && !FUSED ? 512 : 256; }
 template <typename T, int FUSED>

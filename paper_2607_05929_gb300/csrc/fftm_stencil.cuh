@@ -910,7 +910,7 @@ __device__ __forceinline__ void cubic_strain(const double* __restrict__ m36, con
 // Small-strain elastic law of a phase at NP points (c: its law row; an isotropic phase keeps its
 // two constants, fewer products and roundings than the full stiffness).  One branch for the points
 // together: their products interleave and the stiffness is loaded once (the 192^3 FP32 one-pass
-// residual: 226 us, 248 with a branch per point).  The trace's share enters its FMA unrounded: a
+// residual: 228 us; 22 us more with a branch per point).  The trace's share enters its FMA unrounded: a
 // small normal stress beside a large one would else take the rounding of that one's share (D beside
 // a face that the field is cut to zero at: 1.03 to 1.08 times as far from 64 bits).
 template <typename T, int NP>
@@ -1108,7 +1108,8 @@ __device__ __forceinline__ void stress_sym(const ResParams<T>& P, int law, const
 // its gathers, and its general paths (quadratic mean fields, face nodes) would otherwise set the
 // registers of the plain ones: held to four blocks (64 registers) the 128^3 J2 residual measured
 // k_stress 149 -> 112 us, k_stress_inc 144 -> 129, k_div 68 -> 52 / 81 -> 65; three blocks gave
-// 120 / 141 / 56 / 73, five 159 / 141 / 51 / 64.  The hidden latency is worth more than the spills
+// 120 / 141 / 56 / 73, five 159 / 141 / 51 / 64 (all with sums shared between the axes; with the
+// present ones, at four blocks, 121 / 143 / 56 / 65).  The hidden latency is worth more than the spills
 // that four blocks cost (with low parts all 48 corner values of a voxel are alive at once:
 // k_stress_inc stores 440-456 bytes a thread, k_stress with J2 196, k_div's face nodes 40).  The
 // divergence of nine-component stresses (finite strain) gains too: the 128^3 residual of
